@@ -52,30 +52,22 @@ METRIC = "BSSN FP64 point-updates/s (RK4 substeps)"
 UNIT = "point-updates/s"
 
 # FP64 operations (FMA = 2) per interior point of one RHS evaluation (nr_rhs:
-# the k_d1 pre-pass and k_rhs), by workload (the kernel variant it runs), from
-# the kernels' DADD/DMUL/DFMA thread-instruction counts in one ncu capture of
-# that workload's nr_rhs launches: (DADD + DMUL + 2 DFMA) / interior points.  Head-on
-# 256x2x512 (cylindrical, two-point azimuth): k_rhs 215 + 348 + 2 x 1166 = 2895, k_d1 44.3.
-# Head-on with the 8th-order scheme: k_rhs 315 + 408 + 2 x 1517 = 3757, k_d1 122.9.  Large 3D
-# (spherical, general; counted on a 96x48x96 grid of the same kernel): k_rhs 320 + 453 + 2 x 1670 =
-# 4113, k_d1 89.8 (4 FLOP per stored difference, 22.46 differences per point at 384x192x384).
-# Large 3D with the production scheme (the general 8th-order kernel, counted on 96x48x96): k_rhs
-# 489 + 546 + 2 x 2208 = 5451, k_d1 252.2 (11 FLOP per stored difference, 22.93 per point).
-# A workload without a capture reports no FLOP rate.
-F_ALG = {"headon": 2939.3, "large3d": 4202.8, "headon8": 3879.9, "large3d8": 5703.2}
+# the k_d1 pre-pass and k_rhs), by workload (the kernel variant it runs): the FP64 operations of the algorithm
+# as the point code's source has them (add + mul + div + 2 fma, a host census that a test recomputes), with
+# the raw first differences counted as FP64 sums.  The kernels take those, and the advection + dissipation sums
+# (not counted here at all), in integer arithmetic beside the FP64 pipe.
+F_ALG = {"headon": 2294.3, "large3d": 3306.8, "headon8": 2736.9, "large3d8": 4092.2}
 # DRAM bytes (read + write) of the same two launches in that capture; for the large 3D grids the
 # capture's bytes per interior point at 96x48x96 (3275.7 and 5324.5, mostly register-spill lines)
 # times the 28,311,552 points of the full grid
 TRAFFIC = {"headon": 24016384 + 88832 + 94202624 + 510593792,
            "headon8": 24951296 + 119552 + 94502400 + 486498304,
            "large3d": round(3275.7 * 28311552), "large3d8": round(5324.5 * 28311552)}
-# FLOPs of the same right-hand side in the point code's source (a host census of the code those counts
-# were taken from: FMA = 2, one division; without the k_d1 pre-pass); a test recomputes it, so that a
-# change of the kernels' arithmetic cannot leave F_ALG behind unnoticed
-KERNEL_CENSUS = {"headon": 2976, "headon8": 3840, "large3d": 4217, "large3d8": 5590}
+# The same without the k_d1 pre-pass
+KERNEL_CENSUS = {"headon": 2250, "headon8": 2614, "large3d": 3217, "large3d8": 3840}
 # FLOPs over twice the FP64 instructions of the same source (k_d1 + k_rhs): the fraction of the FLOP peak
 # that a fully busy FP64 pipe reaches with this mix (a DADD or DMUL takes an FMA's issue slot for 1 FLOP)
-MIX_CEILING = {"headon": 0.8315, "headon8": 0.8282, "large3d": 0.8345, "large3d8": 0.8272}
+MIX_CEILING = {"headon": 0.7932, "headon8": 0.7765, "large3d": 0.8005, "large3d8": 0.7790}
 # FP64 operations (add + mul + div) per interior point of one RHS evaluation as the oracle's counting
 # build counts them: the plain coordinate-basis evaluation of the same discretisation with generic index
 # loops and the reference metric evaluated at every point -- the work of the method evaluated plainly.
@@ -89,7 +81,7 @@ F_METHOD = {"headon": 28967, "headon8": 49631, "large3d": 28970, "large3d8": 496
 DIAG_FLOPS = {"headon": {"hamiltonian": 1884.0, "momentum": 819.0, "psi4": 3158.0}}
 # the source census of the constraints' point code those counts were taken with (FMA = 2, one division,
 # the square root of |M| not counted: its expansion is most of the 29 FLOP the momentum count adds)
-DIAG_CENSUS = {"headon": {"hamiltonian": 1883, "momentum": 790}}
+DIAG_CENSUS = {"headon": {"hamiltonian": 1881, "momentum": 785}}
 # psi4 modes on the workload's extraction sphere: l <= 8, Gauss-Legendre x uniform nodes
 PSI4_LMAX, PSI4_NTHETA, PSI4_NPHI = 8, 24, 48
 # FP64 pipe of one SM: 2 DFMA per clock (ncu peak_sustained of
@@ -473,7 +465,8 @@ def run_ours(args, spec, world, rank, local):
     if f_alg:
         ach = f_alg * pts / (rhs_ms * 1e-3)
         roof.update(achieved=ach / 1e12, frac=ach / peak, flops_per_point=f_alg,
-                    flops_source="the compiled kernels' DADD + DMUL + 2 DFMA per interior point (ncu)",
+                    flops_source="FP64 operations per interior point in the kernels' source (host census); the "
+                                 "advection + dissipation sums run on the integer pipe and are not counted",
                     mix_ceiling=MIX_CEILING[args.workload])
     else:
         roof.update(achieved=None, frac=None, flops_per_point=None)

@@ -30,6 +30,8 @@
 
 #include <stdint.h>
 
+#include "fixed_sum.cuh"
+
 namespace nrk {
 
 constexpr int NGF = 24;
@@ -37,7 +39,12 @@ enum : int { G_HDD = 0, G_ADD = 6, G_CF = 12, G_TRK = 13, G_LAM = 14, G_VET = 17
 enum : int { FAM_SPH = 0, FAM_CYL = 1 };
 
 // symmetric pair index: (0,0)=0 (0,1)=1 (0,2)=2 (1,1)=3 (1,2)=4 (2,2)=5
-__host__ __device__ constexpr int sp(int i, int j) { return (i > j) ? sp(j, i) : (i == 0 ? j : (i == 1 ? j + 2 : 5)); }
+// (not recursive: a call left in an index when arrays are split into registers keeps the whole array, and every
+// component array of the point code, in local memory; a stack frame of 2.2 KB per thread came from that)
+__host__ __device__ constexpr int sp(int i, int j)
+{
+    return i <= j ? (i == 0 ? j : (i == 1 ? j + 2 : 5)) : (j == 0 ? i : (j == 1 ? i + 2 : 5));
+}
 __host__ __device__ constexpr int spi(int s) { return s < 3 ? 0 : (s < 5 ? 1 : 2); }
 __host__ __device__ constexpr int spj(int s) { return s < 3 ? s : (s < 5 ? s - 2 : 2); }
 __host__ __device__ constexpr bool offd(int s) { return s == 1 || s == 2 || s == 4; }
@@ -215,6 +222,37 @@ __host__ __device__ constexpr int d1slot(int gf)
 }
 __host__ __device__ constexpr int d1gf(int q) { return q < 6 ? q : q == 6 ? G_CF : q == 7 ? G_ALPHA : G_VET + q - 8; }
 
+// Where the raw difference sums of a point come from (template parameter S): differenced inline from the
+// state (0); the mixed differences, and the first differences of the same gridfunctions along axes 0 and 1, from
+// the stored first differences (1); the same with every further first difference, of the state and of the
+// stored differences, taken beforehand on the integer pipe and read from a table (2, 3).  The second
+// differences stay in FP64: along the azimuth near the axis or a pole their rounding, at 2^-53 of f against
+// f'' dxx^2, is multiplied by 1/(dxx S)^2, so another rounding would show in the result.
+// The table lies in the thread's local memory (2) or in shared memory, [entry][lane] (3).
+enum : int { SRC_INLINE = 0, SRC_STORED = 1, SRC_TABLE = 2, SRC_SHARED = 3 };
+template <int S>
+__host__ __device__ constexpr bool src_table() { return S >= SRC_TABLE; }
+template <int S>
+__host__ __device__ constexpr int src_stride() { return S == SRC_SHARED ? 32 : 1; }
+// Table index of each raw sum.  Per gridfunction with second derivatives (d1slot q): the first difference along the
+// last axis (AX < 0: axis 2; else the axis beside 0 and the two-point one), the mixed differences, and f_other -
+// f along a two-point axis; per gridfunction with first derivatives only (lambda 0..2, K: r = 0..3) the
+// first differences.
+template <int AX>
+struct RawIx {
+    static constexpr int NA = AX < 0 ? 3 : 2;        // axes with differences: 0, 1, 2 or 0 and the other one
+    static constexpr int LAST = AX == 2 ? 1 : 2;     // the last of them
+    static constexpr int NM = AX < 0 ? 3 : 1;        // mixed pairs: (0,1), (0,2), (1,2) or (0, LAST)
+    static constexpr int FIRST = N_D1 * (1 + NM), OX = FIRST + 4 * NA, N = OX + (AX < 0 ? 0 : N_D1);
+    __host__ __device__ static constexpr int d1(int q) { return q * (1 + NM); }
+    __host__ __device__ static constexpr int mix(int q, int kl) { return q * (1 + NM) + 1 + (AX < 0 ? (kl == 1 ? 0 : kl == 2 ? 1 : 2) : 0); }
+    __host__ __device__ static constexpr int first(int r, int k) { return FIRST + r * NA + (AX < 0 ? k : (k == 0 ? 0 : 1)); }
+    __host__ __device__ static constexpr int ox(int q) { return OX + q; }
+};
+// r of a gridfunction with first derivatives only
+__host__ __device__ constexpr int f1slot(int gf) { return gf == G_TRK ? 3 : gf - G_LAM; }
+__host__ __device__ constexpr int f1gf(int r) { return r == 3 ? G_TRK : G_LAM + r; }
+
 // sum_k a_k x_k, skipping k = AX where x vanishes (AX is never 0)
 template <int AX>
 __device__ __forceinline__ double dot3(double a0, double a1, double a2, const double x[3])
@@ -228,50 +266,51 @@ __device__ __forceinline__ double dot3(double a0, double a1, double a2, const do
 // ---- frame Hessian of a component function:
 // H_kl f = e_k e_l f - omega^m_kl e_m f  (symmetric in kl); ox is the offset of
 // the other slice of the two-point axis
-// fx, fy: stored first differences of f along axes 0 and 1 (S = true)
-template <int FAM, int KL, int AX, bool S, int ORD>
-__device__ __forceinline__ double hess(const double* f, const double* fx, const double* fy, const long st[3], long ox,
-                                       const Geo& g, const double df[3])
+// fx, fy: stored first differences of f along axes 0 and 1 (S = SRC_STORED); rw: the table (SRC_TABLE, SRC_SHARED) and q
+// the gridfunction's slot in it
+template <int FAM, int KL, int AX, int S, int ORD>
+__device__ __forceinline__ double hess(const double* f, const double* fx, const double* fy, const double* rw, int q,
+                                       const long st[3], long ox, const Geo& g, const double df[3])
 {
+    using R = RawIx<AX>;
     if constexpr (hzero(AX, KL)) return 0.0;
-    if constexpr (KL == 0) return fma(g.D2[0], d2r<ORD>(f, st[0]), -g.d00 * df[0]);
-    if constexpr (KL == 1) return fma(g.DD[0], S ? d1r<ORD>(fx, st[1]) : mixr<ORD>(f, st[0], st[1]), -g.a * df[1]);
-    if constexpr (KL == 2) {
-        const double m = S ? d1r<ORD>(fx, st[2]) : mixr<ORD>(f, st[0], st[2]);
-        if constexpr (FAM == FAM_SPH) return fma(g.DD[1], m, -g.b * df[2]);
-        else return g.DD[1] * m;
-    }
-    if constexpr (KL == 3) {
-        if constexpr (AX == 1) return fma(sc2<FD<ORD>::ax_d2_log2>(g.D2[1]), ld(f + ox) - ld(f), g.a * df[0]);
-        else return fma(g.D2[1], d2r<ORD>(f, st[1]), g.a * df[0]);
-    }
-    if constexpr (KL == 4) {
-        const double m = (S && AX < 0) ? d1r<ORD>(fy, st[2]) : mixr<ORD>(f, st[1], st[2]);
-        if constexpr (FAM == FAM_SPH) return fma(g.DD[2], m, -g.c * df[2]);
-        else return g.DD[2] * m;
-    }
-    if constexpr (KL == 5) {
-        if constexpr (FAM == FAM_SPH) {
-            if constexpr (AX == 2)
-                return fma(sc2<FD<ORD>::ax_d2_log2>(g.D2[2]), ld(f + ox) - ld(f), fma(g.b, df[0], g.c * df[1]));
-            else return fma(g.D2[2], d2r<ORD>(f, st[2]), fma(g.b, df[0], g.c * df[1]));
+    else if constexpr (offd(KL)) {
+        constexpr int k = spi(KL), l = spj(KL);
+        double m;
+        if constexpr (src_table<S>()) m = rw[R::mix(q, KL) * src_stride<S>()];
+        else if constexpr (S == SRC_STORED && k == 0) m = d1r<ORD>(fx, st[l]);
+        else if constexpr (S == SRC_STORED && AX < 0) m = d1r<ORD>(fy, st[l]);
+        else m = mixr<ORD>(f, st[k], st[l]);
+        if constexpr (KL == 1) return fma(g.DD[0], m, -g.a * df[1]);
+        else if constexpr (FAM == FAM_SPH) return fma(g.DD[KL == 2 ? 1 : 2], m, -(KL == 2 ? g.b : g.c) * df[2]);
+        else return g.DD[KL == 2 ? 1 : 2] * m;
+    } else {
+        constexpr int k = spi(KL);
+        double w, m;   // scale and raw second difference
+        if constexpr (AX == k) {
+            w = sc2<FD<ORD>::ax_d2_log2>(g.D2[k]);
+            m = src_table<S>() ? rw[R::ox(q) * src_stride<S>()] : ld(f + ox) - ld(f);
         } else {
-            return fma(g.D2[2], d2r<ORD>(f, st[2]), -g.d22 * df[2]);
+            w = g.D2[k];
+            m = d2r<ORD>(f, st[k]);
         }
+        if constexpr (KL == 0) return fma(w, m, -g.d00 * df[0]);
+        else if constexpr (KL == 3) return fma(w, m, g.a * df[0]);
+        else if constexpr (FAM == FAM_SPH) return fma(w, m, fma(g.b, df[0], g.c * df[1]));
+        else return fma(w, m, -g.d22 * df[2]);
     }
-    return 0.0;
 }
 
-template <int FAM, int AX, bool S, int ORD>
-__device__ __forceinline__ void hess6(const double* f, const double* fx, const double* fy, const long st[3], long ox,
-                                      const Geo& g, const double df[3], double H[6])
+template <int FAM, int AX, int S, int ORD>
+__device__ __forceinline__ void hess6(const double* f, const double* fx, const double* fy, const double* rw, int q,
+                                      const long st[3], long ox, const Geo& g, const double df[3], double H[6])
 {
-    H[0] = hess<FAM, 0, AX, S, ORD>(f, fx, fy, st, ox, g, df);
-    H[1] = hess<FAM, 1, AX, S, ORD>(f, fx, fy, st, ox, g, df);
-    H[2] = hess<FAM, 2, AX, S, ORD>(f, fx, fy, st, ox, g, df);
-    H[3] = hess<FAM, 3, AX, S, ORD>(f, fx, fy, st, ox, g, df);
-    H[4] = hess<FAM, 4, AX, S, ORD>(f, fx, fy, st, ox, g, df);
-    H[5] = hess<FAM, 5, AX, S, ORD>(f, fx, fy, st, ox, g, df);
+    H[0] = hess<FAM, 0, AX, S, ORD>(f, fx, fy, rw, q, st, ox, g, df);
+    H[1] = hess<FAM, 1, AX, S, ORD>(f, fx, fy, rw, q, st, ox, g, df);
+    H[2] = hess<FAM, 2, AX, S, ORD>(f, fx, fy, rw, q, st, ox, g, df);
+    H[3] = hess<FAM, 3, AX, S, ORD>(f, fx, fy, rw, q, st, ox, g, df);
+    H[4] = hess<FAM, 4, AX, S, ORD>(f, fx, fy, rw, q, st, ox, g, df);
+    H[5] = hess<FAM, 5, AX, S, ORD>(f, fx, fy, rw, q, st, ox, g, df);
 }
 // gammabar^kl H_kl (gw: off-diagonal entries doubled), skipping vanishing components
 template <int AX>
@@ -331,6 +370,20 @@ __device__ __forceinline__ void oms(const Geo& g, double s, const double T[6], d
     if constexpr (K == 2 && FAM == FAM_SPH) { j02s(g.b * s, T, o); j12s(g.c * s, T, o); }
 }
 
+// the same with s = 1
+template <int FAM, int K>
+__device__ __forceinline__ void omv(const Geo& g, const double V[3], double o[3])
+{
+    if constexpr (K == 1) j01v(g.a, V, o);
+    if constexpr (K == 2 && FAM == FAM_SPH) { j02v(g.b, V, o); j12v(g.c, V, o); }
+}
+template <int FAM, int K>
+__device__ __forceinline__ void oms(const Geo& g, const double T[6], double o[6])
+{
+    if constexpr (K == 1) j01s(g.a, T, o);
+    if constexpr (K == 2 && FAM == FAM_SPH) { j02s(g.b, T, o); j12s(g.c, T, o); }
+}
+
 __device__ __forceinline__ double gsym(const double m[6], int i, int j) { return m[sp(i, j)]; }
 
 // Inputs of the point evaluation that the kernel precomputes once.
@@ -344,29 +397,32 @@ struct PointIn {
     // NULL where the kernel differences inline
     const double* dx;
     const double* dy;
+    const double* raw;   // the table of raw difference sums (SRC_TABLE, SRC_SHARED)
     Geo g;
 };
 
 // e_k of gridfunction gf: zero along the two-point axis, from the stored first
 // differences where the point has them (S), else inline
-template <int AX, bool S, int ORD>
+template <int AX, int S, int ORD>
 __device__ __forceinline__ double der1(const PointIn& P, int gf, int k)
 {
     if (k == AX) return 0.0;
     const int q = d1slot(gf);
     if (S && q >= 0 && k == 0) return P.g.D[0] * ld(P.dx + (long)q * P.T);
     if (S && AX < 0 && q >= 0 && k == 1) return P.g.D[1] * ld(P.dy + (long)q * P.T);
+    if (src_table<S>())
+        return P.g.D[k] * P.raw[(q >= 0 ? RawIx<AX>::d1(q) : RawIx<AX>::first(f1slot(gf), k)) * src_stride<S>()];
     return P.g.D[k] * d1r<ORD>(P.y + (long)gf * P.T, P.st[k]);
 }
-template <bool S>
+template <int S>
 __device__ __forceinline__ const double* dxp(const PointIn& P, int gf)
 {
-    return S ? P.dx + (long)d1slot(gf) * P.T : nullptr;
+    return S == SRC_STORED ? P.dx + (long)d1slot(gf) * P.T : nullptr;
 }
-template <int AX, bool S>
+template <int AX, int S>
 __device__ __forceinline__ const double* dyp(const PointIn& P, int gf)
 {
-    return (S && AX < 0) ? P.dy + (long)d1slot(gf) * P.T : nullptr;
+    return (S == SRC_STORED && AX < 0) ? P.dy + (long)d1slot(gf) * P.T : nullptr;
 }
 
 // Metric-sector quantities shared by the right-hand side and the
@@ -387,7 +443,7 @@ struct MetricPart {
 // The conformal metric and its inverse, first frame derivatives of h, and
 // Delta (lowered, raised, its trace Delta^k and Delta^k_km): shared by the
 // right-hand side and both constraints.
-template <int FAM, int AX, bool S, int ORD>
+template <int FAM, int AX, int S, int ORD>
 __device__ __forceinline__ void metric_first(const PointIn& P, MetricPart& M)
 {
     static_assert(ax_ok<FAM, AX>(), "two-point axis must be the azimuth");
@@ -431,8 +487,8 @@ __device__ __forceinline__ void metric_first(const PointIn& P, MetricPart& M)
     double Dh[3][6];
 #pragma unroll
     for (int s = 0; s < 6; s++) { Dh[0][s] = dh[0][s]; Dh[1][s] = dh[1][s]; Dh[2][s] = dh[2][s]; }
-    oms<FAM, 1>(g, 1.0, h, Dh[1]);
-    oms<FAM, 2>(g, 1.0, h, Dh[2]);
+    oms<FAM, 1>(g, h, Dh[1]);
+    oms<FAM, 2>(g, h, Dh[2]);
     double (*Dl)[6] = M.Dl;
 #pragma unroll
     for (int k = 0; k < 3; k++)
@@ -474,7 +530,7 @@ __device__ __forceinline__ void metric_first(const PointIn& P, MetricPart& M)
     }
 }
 
-template <int FAM, bool NEED_GH, int AX, bool S, int ORD>
+template <int FAM, bool NEED_GH, int AX, int S, int ORD>
 __device__ __forceinline__ void metric_part(const PointIn& P, MetricPart& M)
 {
     metric_first<FAM, AX, S, ORD>(P, M);
@@ -498,7 +554,7 @@ __device__ __forceinline__ void metric_part(const PointIn& P, MetricPart& M)
     for (int s = 0; s < 6; s++) {
         double df[3] = {dh[0][s], dh[1][s], dh[2][s]};
         double H[6];
-        hess6<FAM, AX, S, ORD>(F(G_HDD + s), dxp<S>(P, G_HDD + s), dyp<AX, S>(P, G_HDD + s), st, P.ox, g, df, H);
+        hess6<FAM, AX, S, ORD>(F(G_HDD + s), dxp<S>(P, G_HDD + s), dyp<AX, S>(P, G_HDD + s), P.raw, d1slot(G_HDD + s), st, P.ox, g, df, H);
         Lh[s] = contract6<AX>(gw, H);
         if constexpr (NEED_GH) {
 #pragma unroll
@@ -542,7 +598,7 @@ __device__ __forceinline__ void metric_part(const PointIn& P, MetricPart& M)
                 X12[s] = fma(cc2, V2[s], fma(g12, h[s], s == 5 ? k22 * Y2[s] : fma(k12, Y1[s], k22 * Y2[s])));
             }
         } else {
-            const double g01 = gi[1] * (g.e0a - g.a * g.a);
+            const double g01 = gi[1] * fma(-g.a, g.a, g.e0a);
             const double a11 = g.a * gi[3];
 #pragma unroll
             for (int s = 0; s < 6; s++) X01[s] = fma(a2, V1[s], fma(g01, h[s], a11 * Y1[s]));
@@ -560,8 +616,8 @@ __device__ __forceinline__ void metric_part(const PointIn& P, MetricPart& M)
     for (int j = 0; j < 3; j++)
 #pragma unroll
         for (int k = 0; k < 3; k++) Dlam[j][k] = der1<AX, S, ORD>(P, G_LAM + k, j);
-    omv<FAM, 1>(g, 1.0, lam, Dlam[1]);
-    omv<FAM, 2>(g, 1.0, lam, Dlam[2]);
+    omv<FAM, 1>(g, lam, Dlam[1]);
+    omv<FAM, 2>(g, lam, Dlam[2]);
     // Quadratic terms. With R[i][m][l] = gammabar^lk Delta^m_ik,
     //   gammabar^kl Delta^m_ki Delta_jml = sum_ml R[i][m][l] Delta_jml   (A_ij; Delta_jml is
     //                                      symmetric in ml, so R is summed over the pair first)
@@ -647,7 +703,7 @@ __device__ __forceinline__ void metric_part(const PointIn& P, MetricPart& M)
     for (int k = 0; k < 3; k++) M.dphi[k] = k == AX ? 0.0 : mhiW * dW[k];
     {
         double HW[6];
-        hess6<FAM, AX, S, ORD>(F(G_CF), dxp<S>(P, G_CF), dyp<AX, S>(P, G_CF), st, P.ox, g, dW, HW);
+        hess6<FAM, AX, S, ORD>(F(G_CF), dxp<S>(P, G_CF), dyp<AX, S>(P, G_CF), P.raw, d1slot(G_CF), st, P.ox, g, dW, HW);
 #pragma unroll
         for (int s = 0; s < 6; s++) {
             // e_i e_j phi = -1/2 W^-1 H_ij W + 2 e_i phi e_j phi; the second term is left out
@@ -659,7 +715,7 @@ __device__ __forceinline__ void metric_part(const PointIn& P, MetricPart& M)
 
 // Output: the 24 right-hand sides without the beta^k d_k advection and
 // without Kreiss-Oliger dissipation (added by the caller, see adv_ko()).
-template <int FAM, int AX, bool S, int ORD>
+template <int FAM, int AX, int S, int ORD>
 __device__ __forceinline__ void rhs_core(const PointIn& P, double eta, double out[NGF])
 {
     const double* y = P.y;
@@ -701,7 +757,7 @@ __device__ __forceinline__ void rhs_core(const PointIn& P, double eta, double ou
     double DDal[6];
     {
         double Hal[6];
-        hess6<FAM, AX, S, ORD>(F(G_ALPHA), dxp<S>(P, G_ALPHA), dyp<AX, S>(P, G_ALPHA), st, P.ox, g, dal, Hal);
+        hess6<FAM, AX, S, ORD>(F(G_ALPHA), dxp<S>(P, G_ALPHA), dyp<AX, S>(P, G_ALPHA), P.raw, d1slot(G_ALPHA), st, P.ox, g, dal, Hal);
 #pragma unroll
         for (int s = 0; s < 6; s++) {
             const double dd = dot3<AX>(Dup[0][s], Dup[1][s], Dup[2][s], dal);
@@ -732,8 +788,8 @@ __device__ __forceinline__ void rhs_core(const PointIn& P, double eta, double ou
     {
         // the generator terms accumulate onto the differences (no additions of zeros)
         double c1[3] = {dvet[1][0], dvet[1][1], dvet[1][2]}, c2[3] = {dvet[2][0], dvet[2][1], dvet[2][2]};
-        omv<FAM, 1>(g, 1.0, vet, c1);
-        omv<FAM, 2>(g, 1.0, vet, c2);
+        omv<FAM, 1>(g, vet, c1);
+        omv<FAM, 2>(g, vet, c2);
 #pragma unroll
         for (int i = 0; i < 3; i++) { Db[i][0] = dvet[0][i]; Db[i][1] = c1[i]; Db[i][2] = c2[i]; }
     }
@@ -749,7 +805,7 @@ __device__ __forceinline__ void rhs_core(const PointIn& P, double eta, double ou
 #pragma unroll
         for (int i = 0; i < 3; i++) {
             double df[3] = {dvet[0][i], dvet[1][i], dvet[2][i]};
-            hess6<FAM, AX, S, ORD>(F(G_VET + i), dxp<S>(P, G_VET + i), dyp<AX, S>(P, G_VET + i), st, P.ox, g, df,
+            hess6<FAM, AX, S, ORD>(F(G_VET + i), dxp<S>(P, G_VET + i), dyp<AX, S>(P, G_VET + i), P.raw, d1slot(G_VET + i), st, P.ox, g, df,
                               Hv[i]);
         }
 #pragma unroll
@@ -856,8 +912,8 @@ __device__ __forceinline__ void rhs_core(const PointIn& P, double eta, double ou
             Q[s] = t;
         }
         double OD[3][3] = {{0, 0, 0}, {0, 0, 0}, {0, 0, 0}};  // (Omega_l Dtr)
-        omv<FAM, 1>(g, 1.0, Dtr, OD[1]);
-        omv<FAM, 2>(g, 1.0, Dtr, OD[2]);
+        omv<FAM, 1>(g, Dtr, OD[1]);
+        omv<FAM, 2>(g, Dtr, OD[2]);
 #pragma unroll
         for (int l = 0; l < 3; l++) {
             double t = DDb[sp(l, 0)][0] + DDb[sp(l, 1)][1];
@@ -922,7 +978,7 @@ __device__ __forceinline__ void rhs_core(const PointIn& P, double eta, double ou
         for (int s = 1; s < 6; s++) trX = fma(gw[s], X[s], trX);
         const double W2 = W * W;
         const double third_trX = trX * (1.0 / 3.0);
-        const double c_div = (-2.0 / 3.0) * divbar + al * K;
+        const double c_div = fma(-2.0 / 3.0, divbar, al * K);
         double r[6];
 #pragma unroll
         for (int s = 0; s < 6; s++) {
@@ -969,7 +1025,7 @@ __device__ __forceinline__ void rhs_core(const PointIn& P, double eta, double ou
             // - lambda^j Dhat_j beta^i + beta^j (Omega_j lambda)^i is added after this block)
             double t = LapB[i];
             t = fma((2.0 / 3.0) * Dvec[i], divbar, t);
-            t = fma((1.0 / 3.0), fma(gsym(gi, i, 2), gdiv[2], fma(gsym(gi, i, 1), gdiv[1], gsym(gi, i, 0) * gdiv[0])), t);
+            t = fma(1.0 / 3.0, fma(gsym(gi, i, 2), gdiv[2], fma(gsym(gi, i, 1), gdiv[1], gsym(gi, i, 0) * gdiv[0])), t);
             // -2 Abar^ij (d_j alpha - 6 alpha d_j phi) - 4/3 alpha gammabar^ij d_j K
             const double v = dot3<AX>(gsym(gi, i, 0), gsym(gi, i, 1), gsym(gi, i, 2), dK);
             t = fma((-4.0 / 3.0) * al, v, t);
@@ -1021,7 +1077,7 @@ template <int FAM, int ORD>
 __device__ __forceinline__ double ham_core(const PointIn& P)
 {
     MetricPart M;
-    metric_part<FAM, false, -1, false, ORD>(P, M);
+    metric_part<FAM, false, -1, SRC_INLINE, ORD>(P, M);
     const double* gi = M.gi;
     const double* gw = M.gw;
     double a[6];
@@ -1061,7 +1117,7 @@ template <int FAM, int ORD>
 __device__ __forceinline__ double mom_core(const PointIn& P, double Mv[3])
 {
     MetricPart M;
-    metric_first<FAM, -1, false, ORD>(P, M);
+    metric_first<FAM, -1, SRC_INLINE, ORD>(P, M);
     const double* y = P.y;
     const long T = P.T;
     const Geo& g = P.g;
@@ -1080,8 +1136,8 @@ __device__ __forceinline__ double mom_core(const PointIn& P, double Mv[3])
         dK[k] = g.D[k] * d1r<ORD>(F(G_TRK), st[k]);
         dphi[k] = (-0.5 * M.iW) * (g.D[k] * d1r<ORD>(F(G_CF), st[k]));
     }
-    oms<FAM, 1>(g, 1.0, a, Da[1]);   // Dhat_k a_ij
-    oms<FAM, 2>(g, 1.0, a, Da[2]);
+    oms<FAM, 1>(g, a, Da[1]);   // Dhat_k a_ij
+    oms<FAM, 2>(g, a, Da[2]);
     double Aud[3][3];  // Abar^k_j
 #pragma unroll
     for (int k = 0; k < 3; k++)
@@ -1113,7 +1169,7 @@ __device__ __forceinline__ double mom_core(const PointIn& P, double Mv[3])
         for (int j = 0; j < 3; j++) {
             // Abar^ij = Abar^i_k gammabar^kj
             const double Auu = fma(Aud[i][2], gsym(gi, 2, j), fma(Aud[i][1], gsym(gi, 1, j), Aud[i][0] * gsym(gi, 0, j)));
-            t = fma(gsym(gi, i, j), fma((-2.0 / 3.0), dK[j], V[j]), fma(6.0 * Auu, dphi[j], t));
+            t = fma(gsym(gi, i, j), fma(-2.0 / 3.0, dK[j], V[j]), fma(6.0 * Auu, dphi[j], t));
         }
         Mv[i] = W2 * t;
     }
@@ -1121,7 +1177,7 @@ __device__ __forceinline__ double mom_core(const PointIn& P, double Mv[3])
 #pragma unroll
     for (int s = 0; s < 6; s++) {
         const int i = spi(s), j = spj(s);
-        const double hm = (offd(s) ? 2.0 : 1.0) * M.h[s] * Mv[i] * Mv[j];
+        const double hm = (offd(s) ? sc2<1>(M.h[s]) : M.h[s]) * Mv[i] * Mv[j];
         q += (i == j) ? fma(Mv[i], Mv[i], hm) : hm;
     }
     return sqrt(q) * M.iW;
@@ -1254,15 +1310,158 @@ __device__ __forceinline__ double advko_apply8(const double* f, const long st[3]
     return k;
 }
 
-// Adds the upwinded advection and the dissipation to the 24 right-hand sides
-// of rhs_core: sigma_metric on the 17 metric gridfunctions (h, a, W, K,
-// lambda), sigma_gauge on the 7 gauge gridfunctions (vet, bet, alpha).
+// beta^k d_k f + dissipation of one gridfunction in FP64 arithmetic: the sums that leave the range of
+// the fixed-point path below (values near the ends of the exponent range, infinities, NaNs)
 template <int AX, int ORD>
-__device__ __forceinline__ void add_adv_ko(const double* y, long T, const long st[3], long ox, const double D[3],
-                                           double sigma_metric, double sigma_gauge, double k[NGF])
+#ifdef __CUDACC__
+__noinline__
+#endif
+__device__ double advko_fp64(const double* f, const long st[3], long ox, const double u[3], const bool fwd[3],
+                             const double D[3], double sigma)
 {
+    if constexpr (ORD == 8) {
+        AdvKoW8 W;
+        advko_weights8<AX>(u, fwd, D, sigma, W);
+        return advko_apply8<AX>(f, st, ox, W, 0.0);
+    } else {
+        AdvKoW W;
+        advko_weights<AX>(u, fwd, D, sigma, W);
+        return advko_apply<AX>(f, st, ox, W, 0.0);
+    }
+}
+
+// Fixed-point scales of the advection + dissipation sum (fixed_sum.cuh).  Per axis the sum is
+// u U + kap K with U and K the integer upwind and dissipation differences, taken exactly.
+//   SH: guard bits of the values; the largest weight sum (4th order: K, 64; 8th: U, 2506) keeps |U|, |K|
+//   within 64 bits (4th) or two 64-bit words (8th, in which S = U, K enters the products as S >> Q);
+//   SC: guard bits of u and kap.
+// With |S >> Q| <= 2^61 and |u|, |kap| < 2^59 no product sum overflows.
+template <int ORD>
+struct FxAdv;
+template <>
+struct FxAdv<4> {
+    static constexpr int G = 3, SH = 2, Q = 0, SC = 6;
+    __host__ __device__ static constexpr int up(int o) { return o == -1 ? -3 : o == 0 ? -10 : o == 1 ? 18 : o == 2 ? -6 : o == 3 ? 1 : 0; }
+    __host__ __device__ static constexpr int ko(int o) { return o == 0 ? -20 : (o == 1 || o == -1) ? 15 : (o == 2 || o == -2) ? -6 : 1; }
+    // along a two-point axis: (a_u u + a_k kap) 2^a_log2 (f_other - f)
+    static constexpr int a_u = 1, a_k = 2, a_log2 = 4;
+};
+template <>
+struct FxAdv<8> {
+    static constexpr int G = 5, SH = 5, Q = 9, SC = 6;
+    __host__ __device__ static constexpr int up(int o)
+    {
+        return o == -3 ? -5 : o == -2 ? 60 : o == -1 ? -420 : o == 0 ? -378 : o == 1 ? 1050 : o == 2 ? -420 : o == 3 ? 140
+             : o == 4 ? -30 : o == 5 ? 3 : 0;
+    }
+    __host__ __device__ static constexpr int ko(int o)
+    {
+        return o == 0 ? -252 : (o == 1 || o == -1) ? 210 : (o == 2 || o == -2) ? -120 : (o == 3 || o == -3) ? 45
+             : (o == 4 || o == -4) ? -10 : 1;
+    }
+    static constexpr int a_u = 3, a_k = 2, a_log2 = 8;
+};
+
+// one axis: U and K of the aligned values v (offsets -G..G from v[0]), as S >> Q
+template <int ORD>
+__device__ __forceinline__ void fx_upko(const fx_i64* v, fx_i64& U, fx_i64& K)
+{
+    using F = FxAdv<ORD>;
+    constexpr int G = F::G;
+    if constexpr (ORD == 4) {
+        U = 0;
+        K = F::ko(0) * v[G];
+#pragma unroll
+        for (int o = 1; o <= G; o++) K += F::ko(o) * (v[G + o] + v[G - o]);
+#pragma unroll
+        for (int o = -G; o <= G; o++)
+            if (F::up(o)) U += F::up(o) * v[G + o];
+    } else {
+        // 64-bit values times up to 11 bits of weight, summed in a high and a low word (which starts at half of what
+        // the shift drops: the sums are rounded, not cut)
+        constexpr fx_i64 half = 1LL << (F::Q - 1);
+        fx_i64 uh = 0, ul = half;
+#pragma unroll
+        for (int o = -G; o <= G; o++)
+            if (F::up(o)) {
+                const FxSplit s = fx_split(v[G + o]);
+                uh += (fx_i64)s.h * F::up(o);
+                ul += (fx_i64)s.l * F::up(o);
+            }
+        const FxSplit c = fx_split(v[G]);
+        fx_i64 kh = (fx_i64)c.h * F::ko(0), kl = (fx_i64)c.l * F::ko(0) + half;
+#pragma unroll
+        for (int o = 1; o <= G; o++) {
+            const FxSplit s = fx_split(v[G + o] + v[G - o]);
+            kh += (fx_i64)s.h * F::ko(o);
+            kl += (fx_i64)s.l * F::ko(o);
+        }
+        U = (uh << (32 - F::Q)) + (ul >> F::Q);
+        K = (kh << (32 - F::Q)) + (kl >> F::Q);
+    }
+}
+
+// the bits of the values of one advection + dissipation sum: centre, offsets -G..G along each axis (strides s),
+// the other slice of a two-point axis
+template <int AX, int ORD>
+struct FxAdvIn {
+    static constexpr int G = FxAdv<ORD>::G;
+    fx_u64 c, o, b[3][2 * G + 1];
+    __device__ __forceinline__ void load(const double* f, const long s[3], long ox)
+    {
+        c = (fx_u64)__double_as_longlong(ld(f));
+        o = AX >= 0 ? (fx_u64)__double_as_longlong(ld(f + ox)) : 0;
+#pragma unroll
+        for (int d = 0; d < 3; d++)
+            if (d != AX)
+#pragma unroll
+                for (int j = -G; j <= G; j++)
+                    if (j) b[d][G + j] = (fx_u64)__double_as_longlong(ld(f + j * s[d]));
+    }
+    __device__ __forceinline__ int key() const   // of the largest value
+    {
+        int k = fx_max(fx_key(c), AX >= 0 ? fx_key(o) : 0);
+#pragma unroll
+        for (int d = 0; d < 3; d++)
+            if (d != AX)
+#pragma unroll
+                for (int j = 0; j <= 2 * G; j++)
+                    if (j != G) k = fx_max(k, fx_key(b[d][j]));
+        return k;
+    }
+    __device__ __forceinline__ bool zero() const
+    {
+        fx_u64 any = c | o;
+#pragma unroll
+        for (int d = 0; d < 3; d++)
+            if (d != AX)
+#pragma unroll
+                for (int j = 0; j <= 2 * G; j++)
+                    if (j != G) any |= b[d][j];
+        return !(any << 1);
+    }
+};
+
+// The upwinded advection and the dissipation of the 24 gridfunctions: sigma_metric on the 17 metric
+// gridfunctions (h, a, W, K, lambda), sigma_gauge on the 7 gauge gridfunctions (vet, bet, alpha).
+// Gridfunctions first, first + step, ..., gridfunction g into sum[g * stride].
+// Each gridfunction is one loop pass on the integer pipe: its values are aligned, differenced exactly along each
+// axis (mirrored where the shift is not positive, so the upwind weights are the same), multiplied by
+// u = |vet^d| D_d and kap (fixed-point numbers on the point's largest exponent) and summed exactly; the
+// result is rounded once.
+template <int AX, int ORD>
+__device__ __forceinline__ void adv_ko_sums(const double* y, long T, const long st[3], long ox, const double D[3],
+                                            double sigma_metric, double sigma_gauge, double* sum, int stride = 1,
+                                            int first = 0, int step = 1)
+{
+    using F = FxAdv<ORD>;
+    constexpr int G = F::G;
+    constexpr double kc = ORD == 8 ? 0.8203125 : 0.1875;   // D_d / (S_d dxx_d): 840/1024 or 12/64
     double u[3];
     bool fwd[3];
+    fx_u64 ub[3], kb[2][3];
+    long s[3];
+    int key = 0;
 #pragma unroll
     for (int d = 0; d < 3; d++) {
         const double v = ld(y + (long)(G_VET + d) * T);
@@ -1270,20 +1469,197 @@ __device__ __forceinline__ void add_adv_ko(const double* y, long T, const long s
         // v > 0 by the sign of the bit pattern, on the integer pipe: the same answer for
         // every value but NaN (+0 and -0 both give the backward stencil)
         fwd[d] = __double_as_longlong(v) > 0;
+        s[d] = fwd[d] ? st[d] : -st[d];
+        ub[d] = (fx_u64)__double_as_longlong(u[d]);
+        kb[0][d] = (fx_u64)__double_as_longlong(kc * sigma_metric * D[d]);
+        kb[1][d] = (fx_u64)__double_as_longlong(kc * sigma_gauge * D[d]);
+        key = fx_max(key, fx_max(fx_key(ub[d]), fx_max(fx_key(kb[0][d]), fx_key(kb[1][d]))));
     }
-    if constexpr (ORD == 8) {
-        AdvKoW8 Wm, Wg;
-        advko_weights8<AX>(u, fwd, D, sigma_metric, Wm);
-        advko_weights8<AX>(u, fwd, D, sigma_gauge, Wg);
+    const int Ec = key >> 20;
+    FxSplit cu[3], ck[2][3];
 #pragma unroll
-        for (int g = 0; g < NGF; g++) k[g] = advko_apply8<AX>(y + (long)g * T, st, ox, g < G_VET ? Wm : Wg, k[g]);
-    } else {
-        AdvKoW Wm, Wg;
-        advko_weights<AX>(u, fwd, D, sigma_metric, Wm);
-        advko_weights<AX>(u, fwd, D, sigma_gauge, Wg);
-#pragma unroll
-        for (int g = 0; g < NGF; g++) k[g] = advko_apply<AX>(y + (long)g * T, st, ox, g < G_VET ? Wm : Wg, k[g]);
+    for (int d = 0; d < 3; d++) {
+        if (d == AX) {
+            const fx_i64 uu = fx_in<F::SC>(ub[d], Ec);
+            cu[d].h = cu[d].l = 0;
+            ck[0][d] = fx_split(F::a_u * uu + F::a_k * fx_in<F::SC>(kb[0][d], Ec));
+            ck[1][d] = fx_split(F::a_u * uu + F::a_k * fx_in<F::SC>(kb[1][d], Ec));
+            continue;
+        }
+        cu[d] = fx_split(fx_in<F::SC>(ub[d], Ec));
+        ck[0][d] = fx_split(fx_in<F::SC>(kb[0][d], Ec));
+        ck[1][d] = fx_split(fx_in<F::SC>(kb[1][d], Ec));
     }
+    // the values' exponents for which no intermediate or result leaves the normal range
+    const bool okc = Ec >= 64 && Ec < 2047;
+    const int elo = fx_max(64, 1150 - Ec), ehi = 3000 - Ec < 2046 ? 3000 - Ec : 2046;
+    // the values of the next gridfunction are loaded while one is summed, where the registers hold both
+    constexpr bool AHEAD = (2 * G + 1) * (AX < 0 ? 3 : 2) <= 24;
+    FxAdvIn<AX, ORD> in, next;
+    if (AHEAD) in.load(y + (long)first * T, s, ox);
+#ifdef __CUDACC__
+#pragma unroll 1
+#endif
+    for (int g = first; g < NGF; g += step) {
+        const double* f = y + (long)g * T;
+        if (AHEAD) {
+            if (g + step < NGF) next.load(f + step * T, s, ox);
+        } else {
+            in.load(f, s, ox);
+        }
+        const int E = in.key() >> 20;
+        double r;
+        if (okc && E >= elo && E <= ehi) {
+            const fx_i64 vc = fx_in<F::SH>(in.c, E);
+            FxDot dot = {0, 0};
+#pragma unroll
+            for (int d = 0; d < 3; d++) {
+                const FxSplit kap = g < G_VET ? ck[0][d] : ck[1][d];
+                if (d == AX) {
+                    const fx_i64 w = fx_in<F::SH>(in.o, E) - vc;
+                    fx_mac(dot, kap, fx_split(F::a_log2 >= F::Q ? w << (F::a_log2 >= F::Q ? F::a_log2 - F::Q : 0)
+                                                                : w >> (F::Q >= F::a_log2 ? F::Q - F::a_log2 : 0)));
+                    continue;
+                }
+                fx_i64 v[2 * G + 1], U, K;
+#pragma unroll
+                for (int o = -G; o <= G; o++) v[G + o] = o ? fx_in<F::SH>(in.b[d][G + o], E) : vc;
+                fx_upko<ORD>(v, U, K);
+                fx_mac(dot, cu[d], fx_split(U));
+                fx_mac(dot, kap, fx_split(K));
+            }
+            r = fx_out2(dot.hh, dot.cross, E + Ec - 2 * 1075 - F::SH - F::SC + F::Q + 32);
+        } else if (okc && in.zero()) {
+            r = 0.0;   // all values zero: the sum is zero for any finite weights
+        } else {
+            r = advko_fp64<AX, ORD>(f, st, ox, u, fwd, D, g < G_VET ? sigma_metric : sigma_gauge);
+        }
+        sum[g * stride] = r;
+        if (AHEAD) in = next;
+    }
+}
+
+// the raw first difference in FP64: sums that leave the range of fx_d1
+template <int ORD>
+#ifdef __CUDACC__
+__noinline__
+#endif
+__device__ double d1_fp64(const double* f, long s)
+{
+    return d1r<ORD>(f, s);
+}
+
+// The raw first difference of f along stride s, exact up to the alignment of the values to the largest of them and
+// rounded once.  4th order: a sum within 64 bits (weights up to 18 in all, 5 guard bits); 8th order: in two
+// words (weights up to 1750, 9 guard bits).  load() reads the values, sum() adds them up.
+template <int ORD>
+struct FxD1 {
+    static constexpr int M = FD<ORD>::M, SH = ORD == 4 ? 5 : 9;
+    const double* f;
+    long s;
+    fx_u64 b[2 * M];   // offsets -M..-1, 1..M
+    __device__ __forceinline__ void load()
+    {
+#pragma unroll
+        for (int j = 0; j < 2 * M; j++) b[j] = (fx_u64)__double_as_longlong(ld(f + (j < M ? j - M : j - M + 1) * s));
+    }
+    __device__ __forceinline__ double sum() const
+    {
+        int k = 0;
+#pragma unroll
+        for (int j = 0; j < 2 * M; j++) k = fx_max(k, fx_key(b[j]));
+        const int E = k >> 20;
+        if (E >= 128 && E <= 2000) {
+            fx_i64 d[M];   // f(+o) - f(-o), o = 1..M
+#pragma unroll
+            for (int o = 1; o <= M; o++) d[o - 1] = fx_in<SH>(b[M + o - 1], E) - fx_in<SH>(b[M - o], E);
+            if constexpr (ORD == 4) {
+                return fx_out(8 * d[0] - d[1], E - 1075 - SH);
+            } else {
+                constexpr int w[4] = {672, -168, 32, -3};
+                fx_i64 h = 0, l = 0;
+#pragma unroll
+                for (int o = 0; o < M; o++) {
+                    const FxSplit m = fx_split(d[o]);
+                    h += (fx_i64)m.h * w[o];
+                    l += (fx_i64)m.l * w[o];
+                }
+                return fx_out2(h, l, E - 1075 - SH);
+            }
+        }
+        fx_u64 any = 0;
+#pragma unroll
+        for (int j = 0; j < 2 * M; j++) any |= b[j];
+        return any << 1 ? d1_fp64<ORD>(f, s) : 0.0;
+    }
+};
+
+// a - b, rounded as the FP64 subtraction rounds it
+__device__ __forceinline__ double fx_sub(double a, double b)
+{
+    const fx_u64 ba = (fx_u64)__double_as_longlong(a), bb = (fx_u64)__double_as_longlong(b);
+    const int E = fx_max(fx_key(ba), fx_key(bb)) >> 20;
+    if (E >= 128 && E <= 2000) return fx_out(fx_in<9>(ba, E) - fx_in<9>(bb, E), E - 1075 - 9);
+    return a - b;
+}
+
+// The table of raw difference sums of one point (RawIx); d1x and d1y: the stored first differences at this
+// point (k_d1).  Rolled loops (the code must stay in the instruction cache beside the FP64 part), each entry's
+// values loaded while the one before is summed.  Entries first, first + step, ... of both parts, entry j into raw[j * stride].
+template <int AX, int ORD>
+__device__ __forceinline__ void raw_table(const double* y, const double* d1x, const double* d1y, long T, const long st[3],
+                                          long ox, double* raw, int stride = 1, int first = 0, int step = 1)
+{
+    using R = RawIx<AX>;
+    auto entry = [&](int j) {
+        FxD1<ORD> e;
+        e.s = st[R::LAST];
+        if (j < R::FIRST) {
+            const int q = j / (1 + R::NM), m = j % (1 + R::NM);
+            e.f = m == 0 ? y + (long)d1gf(q) * T : (m == 3 ? d1y : d1x) + (long)q * T;
+            if (AX < 0 && m == 1) e.s = st[1];
+        } else {
+            const int r = (j - R::FIRST) / R::NA, a = (j - R::FIRST) % R::NA;
+            e.f = y + (long)f1gf(r) * T;
+            if (a == 0) e.s = st[0];
+            else if (AX < 0 && a == 1) e.s = st[1];
+        }
+        e.load();
+        return e;
+    };
+    FxD1<ORD> e = entry(first);
+#ifdef __CUDACC__
+#pragma unroll 1
+#endif
+    for (int j = first; j < R::OX; j += step) {
+        const FxD1<ORD> next = entry(j + step < R::OX ? j + step : j);
+        raw[j * stride] = e.sum();
+        e = next;
+    }
+    if constexpr (AX >= 0) {
+        double o = ld(y + (long)d1gf(first) * T + ox), c = ld(y + (long)d1gf(first) * T);
+#ifdef __CUDACC__
+#pragma unroll 1
+#endif
+        for (int q = first; q < N_D1; q += step) {
+            const double* f = y + (long)d1gf(q + step < N_D1 ? q + step : q) * T;
+            const double on = ld(f + ox), cn = ld(f);
+            raw[R::ox(q) * stride] = fx_sub(o, c);
+            o = on;
+            c = cn;
+        }
+    }
+}
+
+// Adds the upwinded advection and the dissipation to the 24 right-hand sides of rhs_core.
+template <int AX, int ORD>
+__device__ __forceinline__ void add_adv_ko(const double* y, long T, const long st[3], long ox, const double D[3],
+                                           double sigma_metric, double sigma_gauge, double k[NGF])
+{
+    double sum[NGF];
+    adv_ko_sums<AX, ORD>(y, T, st, ox, D, sigma_metric, sigma_gauge, sum);
+#pragma unroll
+    for (int g = 0; g < NGF; g++) k[g] += sum[g];
 }
 
 }  // namespace nrk

@@ -81,6 +81,7 @@ int build_table(nr_batch* b, const double* dts, bool ssp)
         B.finf = g->finf;
         B.wspeed = g->wspeed;
         B.n_outer = g->n_outer;
+        B.tx = ts.tx;
         B.tiles_x = (g->K.N0 + ts.tx - 1) / ts.tx;
         const int tiles_y = (g->K.N1 * g->K.N2 + ts.ty - 1) / ts.ty;
         B.w_begin = w;

@@ -2,13 +2,11 @@
 // launch helpers, instantiated once per coordinate family and finite-difference
 // order (nr_batch_{sph,cyl}{,8}.cu) so the four compile in parallel.
 //
-// A work item is either a TX x TY tile of one grid's interior points or a
-// chunk of TX*TY of its pure-outer ghost points.  One launch per RK substage
-// covers the items of all grids, one block per item: the block finds its grid
+// A work item is either a tx x ty tile of one grid's interior points or a chunk of tx * ty of its
+// pure-outer ghost points.  One launch per RK substage covers the items of all grids, one block of
+// tx * ty threads per item: the block finds its grid
 // by binary search over the items' start indices and stages that grid's
-// record in shared memory.  (A persistent variant that took items from an
-// atomic counter carried its loop state through the 255-register point code
-// and spilled three to four times as much.)  Every
+// record in shared memory.  Every
 // point runs the same per-point code as the single-grid kernels
 // (nr_stage.cuh, with the same two-point-azimuth specialisation AX; the grids
 // of one batch share it), so a grid's state after n batched steps is bitwise
@@ -30,11 +28,13 @@ struct __align__(16) BGrid {
     const double* finf;
     const double* wspeed;
     int n_outer;
-    int tiles_x;
+    int tiles_x, tx;           // tiles of tx columns, blockDim.x points
     int w_begin, w_rhs_end, w_end;
     int ssp;                   // the table's integrator: 0 RK4 (st[0..3]), 1 SSPRK3 (st[0..2])
     Stage st[4];
 };
+
+constexpr int BATCH_MAX_THREADS = 128, BATCH_MIN_BLOCKS = 4;
 
 struct BInner {
     int grid, dst, src, negmask;
@@ -53,9 +53,9 @@ __device__ __forceinline__ void stage_buffers(const BGrid& B, int stage, const d
     }
 }
 
-template <int FAM, int AX, int ORD, int TX, int TY>
-__global__ void __launch_bounds__(TX* TY) k_batch_stage(const BGrid* __restrict__ grids, int ngrids, int total,
-                                                         int stage)
+template <int FAM, int AX, int ORD>
+__global__ void __launch_bounds__(BATCH_MAX_THREADS, BATCH_MIN_BLOCKS) k_batch_stage(const BGrid* __restrict__ grids,
+                                                                                      int ngrids, int total, int stage)
 {
     // one block per work item; the item's grid record is staged in shared memory
     __shared__ __align__(16) unsigned long long s_grid[(sizeof(BGrid) + 7) / 8];
@@ -70,7 +70,7 @@ __global__ void __launch_bounds__(TX* TY) k_batch_stage(const BGrid* __restrict_
     }
     {
         const unsigned long long* src = reinterpret_cast<const unsigned long long*>(grids + lo);
-        for (int q = tid; q < (int)(sizeof(BGrid) / 8); q += TX * TY) s_grid[q] = src[q];
+        for (int q = tid; q < (int)(sizeof(BGrid) / 8); q += blockDim.x) s_grid[q] = src[q];
     }
     __syncthreads();
     const BGrid& B = *reinterpret_cast<const BGrid*>(s_grid);
@@ -79,13 +79,13 @@ __global__ void __launch_bounds__(TX* TY) k_batch_stage(const BGrid* __restrict_
     double* out;
     stage_buffers(B, stage, yin, out, yn);
     if (w < B.w_rhs_end) {
-        const int t = w - B.w_begin;
-        const int i = (t % B.tiles_x) * TX + tid % TX;
-        const int j = (t / B.tiles_x) * TY + tid / TX;
+        const int t = w - B.w_begin, ty = (int)blockDim.x / B.tx;
+        const int i = (t % B.tiles_x) * B.tx + tid % B.tx;
+        const int j = (t / B.tiles_x) * ty + tid / B.tx;
         if (i < B.K.N0 && j < B.K.N1 * B.K.N2)
-            rhs_point_stage<FAM, AX, true, ORD>(B.K, yin, B.d1x, B.d1y, out, yn, B.acc, B.st[stage], i, j);
+            rhs_point_stage<FAM, AX, ORD>(B.K, yin, B.d1x, B.d1y, out, yn, B.acc, B.st[stage], i, j);
     } else {
-        const int p = (w - B.w_rhs_end) * (TX * TY) + tid;
+        const int p = (w - B.w_rhs_end) * (int)blockDim.x + tid;
         if (p < B.n_outer)
             outer_point_stage<FAM, ORD, ssp_first_short<AX>()>(B.K, B.outer[p], yin, out, yn, B.acc, B.finf, B.wspeed,
                                                                B.st[stage]);
@@ -112,17 +112,17 @@ __global__ void __launch_bounds__(256) k_batch_d1(const BGrid* __restrict__ grid
     d1_point<AX, ORD>(B.K, yin, B.d1x, B.d1y, (long)(w - B.d1_begin) * 256 + threadIdx.x);
 }
 
-// tile shapes the autotuner tries (threads per block = TX * TY)
+// tile shapes the autotuner tries
 struct TileShape {
     int tx, ty;
 };
 constexpr TileShape kTiles[] = {{32, 4}, {64, 2}, {128, 1}, {16, 8}, {32, 2}, {64, 1}, {32, 1}};
 constexpr int kNumTiles = sizeof(kTiles) / sizeof(kTiles[0]);
 
-template <int FAM, int AX, int ORD, int TX, int TY>
-cudaError_t launch_bstage(const BGrid* g, int n, int total, int stage, cudaStream_t s)
+template <int FAM, int AX, int ORD>
+cudaError_t launch_bstage(int tile, const BGrid* g, int n, int total, int stage, cudaStream_t s)
 {
-    if (total > 0) k_batch_stage<FAM, AX, ORD, TX, TY><<<total, TX * TY, 0, s>>>(g, n, total, stage);
+    if (total > 0) k_batch_stage<FAM, AX, ORD><<<total, kTiles[tile].tx * kTiles[tile].ty, 0, s>>>(g, n, total, stage);
     return cudaGetLastError();
 }
 
@@ -131,20 +131,6 @@ cudaError_t launch_batch_d1(const BGrid* g, int n, int total_d1, int stage, cuda
 {
     if (total_d1 > 0) k_batch_d1<AX, ORD><<<total_d1, 256, 0, s>>>(g, n, total_d1, stage);
     return cudaGetLastError();
-}
-
-template <int FAM, int AX, int ORD>
-cudaError_t dispatch_stage(int tile, const BGrid* g, int n, int total, int stage, cudaStream_t s)
-{
-    switch (tile) {
-    case 0: return launch_bstage<FAM, AX, ORD, 32, 4>(g, n, total, stage, s);
-    case 1: return launch_bstage<FAM, AX, ORD, 64, 2>(g, n, total, stage, s);
-    case 2: return launch_bstage<FAM, AX, ORD, 128, 1>(g, n, total, stage, s);
-    case 3: return launch_bstage<FAM, AX, ORD, 16, 8>(g, n, total, stage, s);
-    case 4: return launch_bstage<FAM, AX, ORD, 32, 2>(g, n, total, stage, s);
-    case 5: return launch_bstage<FAM, AX, ORD, 64, 1>(g, n, total, stage, s);
-    default: return launch_bstage<FAM, AX, ORD, 32, 1>(g, n, total, stage, s);
-    }
 }
 
 // one translation unit per family and order (nr_batch_{sph,cyl}{,8}.cu) defines, through
@@ -163,8 +149,8 @@ NRK_BATCH_DECL(cyl8)
     cudaError_t batch_stage_##NAME(bool two_point, int tile, const BGrid* g, int n, int total, int stage,      \
                                    cudaStream_t s)                                                             \
     {                                                                                                          \
-        return two_point ? dispatch_stage<FAM_, AXTWO_, ORD_>(tile, g, n, total, stage, s)                     \
-                         : dispatch_stage<FAM_, -1, ORD_>(tile, g, n, total, stage, s);                        \
+        return two_point ? launch_bstage<FAM_, AXTWO_, ORD_>(tile, g, n, total, stage, s)                      \
+                         : launch_bstage<FAM_, -1, ORD_>(tile, g, n, total, stage, s);                         \
     }                                                                                                          \
     cudaError_t batch_d1_##NAME(bool two_point, const BGrid* g, int n, int total_d1, int stage, cudaStream_t s) \
     {                                                                                                          \

@@ -48,6 +48,17 @@ __device__ __forceinline__ Geo make_geo(const GridK& G, int i0, int i1, int i2)
     return g;
 }
 
+// Geo::D alone: 1/(den1 dxx_k S_k)
+template <int FAM>
+__device__ __forceinline__ void make_geo_scales(const GridK& G, int i0, int i1, int i2, double D[3])
+{
+    const double* A0 = G.rfm.ax0;
+    const double a = ld(A0 + G.n0 + i0);
+    D[0] = ld(A0 + i0) * G.inv_d1[0];
+    D[1] = a * G.inv_d1[1];
+    D[2] = (FAM == FAM_SPH ? a * ld(G.rfm.ax1 + i1) : ld(G.rfm.ax2 + i2)) * G.inv_d1[2];
+}
+
 __device__ __forceinline__ void cart_of(const GridK& G, int i0, int i1, int i2, double x[3])
 {
     if (G.fam == FAM_SPH) {

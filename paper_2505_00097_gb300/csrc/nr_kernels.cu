@@ -19,8 +19,6 @@
 #include <math.h>
 
 #include <algorithm>
-#include <atomic>
-#include <mutex>
 
 #include "bssn_point.cuh"
 #include "nr_geo.cuh"
@@ -28,8 +26,6 @@
 #include "nr_stage.cuh"
 
 namespace nrk {
-
-constexpr int RHS_BX = 32, RHS_BY = 4;
 
 // Raw first differences along axis 0 (and, on a general grid, axis 1) of the N_D1
 // gridfunctions with second derivatives, at interior i0 and every row a mixed
@@ -42,98 +38,78 @@ __global__ void __launch_bounds__(256) k_d1(GridK G, const double* __restrict__ 
     d1_point<AX, ORD>(G, y, d1x, d1y, (long)blockIdx.x * blockDim.x + threadIdx.x);
 }
 
-// one tile of k_rhs: tile tb < oa.nblocks takes pure-outer points, 128 each; the others tile
-// (i0, j = i1 + N1 i2) in 32 x 4 points
+// One RK stage (or, MODE_RHS, the right-hand side alone), one point per thread: the first oa.nblocks blocks take
+// the pure-outer points, the others tile (i0, j = i1 + N1 i2) in 32 x RHS_BY points.
+//
+// Bound: the FP64 pipe (2 lanes a cycle per SM: 16 to 20 cycles per warp instruction), with the difference sums on the
+// integer pipe beside it (fixed_sum.cuh).  A warp does its integer passes first and its FP64 part after
+// them; four warps per scheduler (128 registers, 3 to 5 KB of spills) keep one of them in its FP64 part nearly
+// always: 681 us per right-hand side on 256x2x512, against 693 us with three (168 registers) and 746 us with two (255
+// registers, no spills); all in FP64 arithmetic, two per scheduler: 864 us.  8th order on the same grid: 1137 -> 814
+// us; 192x96x192 spherical: 15.66 -> 11.68 ms (4th), 23.2 -> 14.5 ms (8th).
+constexpr int RHS_BY = 4;
 template <int FAM, int AX, int ORD>
-__device__ __forceinline__ void rhs_tile(const GridK& G, const double* __restrict__ yin, const double* __restrict__ d1x,
-                                         const double* __restrict__ d1y, double* out, const double* yn, double* acc,
-                                         const Stage& st, const OuterArgs& oa, int tb, int nbx)
+__global__ void __launch_bounds__(32 * RHS_BY, 4)
+    k_rhs(GridK G, const double* __restrict__ yin, const double* __restrict__ d1x, const double* __restrict__ d1y,
+          double* out, const double* yn, double* acc, Stage st, OuterArgs oa)
 {
-    if (tb < oa.nblocks) {
-        const int t = tb * (RHS_BX * RHS_BY) + threadIdx.y * RHS_BX + threadIdx.x;
+    if ((int)blockIdx.x < oa.nblocks) {
+        const int t = blockIdx.x * (32 * RHS_BY) + threadIdx.y * 32 + threadIdx.x;
         if (t < oa.npts)
             outer_point_stage<FAM, ORD, ssp_first_short<AX>()>(G, oa.pts[t], yin, out, yn, acc, oa.finf, oa.wspeed, st);
         return;
     }
-    const int b = tb - oa.nblocks;
-    const int i = (b % nbx) * RHS_BX + threadIdx.x;
-    const int j = (b / nbx) * RHS_BY + threadIdx.y;
-    if (i < G.N0 && j < G.N1 * G.N2) rhs_point_stage<FAM, AX, true, ORD>(G, yin, d1x, d1y, out, yn, acc, st, i, j);
+    const int b = blockIdx.x - oa.nblocks, nbx = (G.N0 + 31) / 32;
+    const int i = (b % nbx) * 32 + threadIdx.x, j = (b / nbx) * RHS_BY + threadIdx.y;
+    if (i < G.N0 && j < G.N1 * G.N2) rhs_point_stage<FAM, AX, ORD>(G, yin, d1x, d1y, out, yn, acc, st, i, j);
 }
 
-// Whether k_rhs runs a grid of the resident blocks, each striding over the tiles (every warp then
-// keeps its slot for the whole launch): measured faster for the two-point-azimuth kernels; the
-// general kernels, whose loop adds register spills, run one block per tile
-template <int AX>
-__host__ __device__ constexpr bool rhs_strided()
+// The same for grids of few points, whose time is one warp's way through its tile: a block of SPREAD_WARPS warps
+// takes 32 consecutive interior points (i0 fastest) and divides the integer passes among its warps.  64x16x2: 93
+// -> 68 us; 72x12x24: 196 -> 168 us (with k_d1 and the launches; the all-FP64 kernel took 83 and 196 us).
+// Three blocks per SM (168 registers): two are 3 % faster on the smallest grids and 35 % slower on 72x12x24, four 6
+// and 9 % slower.  It is taken up to SPREAD_TILES tiles, two rounds of three blocks on each of 152 SMs (864 tiles: 178 against 197
+// us); at 8,192 tiles it is half as fast as k_rhs, whose four warps share the FP64 pipe.
+constexpr long SPREAD_TILES = 2 * 3 * 152;
+template <int FAM, int AX, int ORD>
+__global__ void __launch_bounds__(32 * SPREAD_WARPS, 3)
+    k_rhs_spread(GridK G, const double* __restrict__ yin, const double* __restrict__ d1x,
+                 const double* __restrict__ d1y, double* out, const double* yn, double* acc, Stage st, OuterArgs oa)
 {
-    return AX >= 0;
+    __shared__ double tab[RawIx<AX>::N + NGF][32];
+    __shared__ int slot;
+    if ((int)blockIdx.x < oa.nblocks) {
+        const int t = blockIdx.x * (32 * SPREAD_WARPS) + threadIdx.x;
+        if (t < oa.npts)
+            outer_point_stage<FAM, ORD, ssp_first_short<AX>()>(G, oa.pts[t], yin, out, yn, acc, oa.finf, oa.wspeed, st);
+        return;
+    }
+    // the blocks of one SM put their FP64 warps on different schedulers (warp slots modulo 4)
+    if (threadIdx.x == 0) {
+        unsigned w;
+        asm volatile("mov.u32 %0, %%warpid;" : "=r"(w));
+        slot = (w / SPREAD_WARPS) % SPREAD_WARPS;
+    }
+    __syncthreads();
+    const int n = G.N0 * G.N1 * G.N2, p = (blockIdx.x - oa.nblocks) * 32 + (threadIdx.x & 31), q = p < n ? p : n - 1;
+    rhs_spread_stage<FAM, AX, ORD>(G, yin, d1x, d1y, out, yn, acc, st, q % G.N0, q / G.N0, p < n, threadIdx.x / 32,
+                                   slot, tab);
 }
 
 template <int FAM, int AX, int ORD>
-__global__ void __launch_bounds__(RHS_BX* RHS_BY) k_rhs(GridK G, const double* __restrict__ yin,
-                                                        const double* __restrict__ d1x, const double* __restrict__ d1y,
-                                                        double* out, const double* yn, double* acc, Stage st,
-                                                        OuterArgs oa)
+cudaError_t launch_k_rhs(cudaStream_t s, const GridK& G, const double* yin, double* d1x, double* d1y, double* out,
+                         const double* yn, double* acc, const Stage& st, OuterArgs oa)
 {
-    const int nbx = (G.N0 + RHS_BX - 1) / RHS_BX;
-    if constexpr (rhs_strided<AX>()) {
-        const int ntiles = oa.nblocks + nbx * ((G.N1 * G.N2 + RHS_BY - 1) / RHS_BY);
-#pragma unroll 1
-        for (int tb = (int)blockIdx.x; tb < ntiles; tb += (int)gridDim.x)
-            rhs_tile<FAM, AX, ORD>(G, yin, d1x, d1y, out, yn, acc, st, oa, tb, nbx);
+    const long tiles = ((long)G.N0 * G.N1 * G.N2 + 31) / 32;
+    if (tiles <= SPREAD_TILES) {
+        oa.nblocks = (oa.npts + 32 * SPREAD_WARPS - 1) / (32 * SPREAD_WARPS);
+        k_rhs_spread<FAM, AX, ORD><<<(unsigned)(tiles + oa.nblocks), 32 * SPREAD_WARPS, 0, s>>>(G, yin, d1x, d1y, out, yn,
+                                                                                              acc, st, oa);
     } else {
-        rhs_tile<FAM, AX, ORD>(G, yin, d1x, d1y, out, yn, acc, st, oa, (int)blockIdx.x, nbx);
+        oa.nblocks = (oa.npts + 32 * RHS_BY - 1) / (32 * RHS_BY);
+        const long nb = (long)((G.N0 + 31) / 32) * (((long)G.N1 * G.N2 + RHS_BY - 1) / RHS_BY) + oa.nblocks;
+        k_rhs<FAM, AX, ORD><<<(unsigned)nb, dim3(32, RHS_BY), 0, s>>>(G, yin, d1x, d1y, out, yn, acc, st, oa);
     }
-}
-
-// k_rhs blocks resident on the whole device, per instantiation (family x azimuth axis x order), by
-// device; 0: not yet known (a launch then runs one block per tile).  Filled by rhs_kernels_init.
-constexpr int RHS_MAX_DEV = 64;
-constexpr int RHS_VARIANTS = 8;
-std::atomic<int> g_rhs_resident[RHS_MAX_DEV][RHS_VARIANTS];
-std::mutex g_rhs_mu;
-
-template <int FAM, int AX, int ORD>
-constexpr int rhs_variant()
-{
-    return (FAM == FAM_SPH ? 0 : 4) + (AX < 0 ? 0 : 2) + (ORD == 8 ? 1 : 0);
-}
-
-template <int FAM, int AX, int ORD>
-cudaError_t rhs_init_one(int dev, int nsm)
-{
-    int occ = 0;
-    const cudaError_t e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&occ, k_rhs<FAM, AX, ORD>, RHS_BX * RHS_BY, 0);
-    if (e != cudaSuccess) return e;
-    g_rhs_resident[dev][rhs_variant<FAM, AX, ORD>()].store(occ * nsm);
-    return cudaSuccess;
-}
-
-template <int FAM, int AX, int ORD>
-int rhs_resident()
-{
-    int dev = 0;
-    if (cudaGetDevice(&dev) != cudaSuccess || dev < 0 || dev >= RHS_MAX_DEV) return 0;
-    return g_rhs_resident[dev][rhs_variant<FAM, AX, ORD>()].load();
-}
-
-template <int FAM, int AX, int ORD>
-cudaError_t launch_k_rhs(long nb, cudaStream_t s, const GridK& G, const double* yin, double* d1x, double* d1y,
-                         double* out, const double* yn, double* acc, const Stage& st, const OuterArgs& oa)
-{
-    int res = rhs_resident<FAM, AX, ORD>();
-    if (res == 0) {
-        // first launch on this device outside a stream capture: fill the table now
-        cudaStreamCaptureStatus cs = cudaStreamCaptureStatusNone;
-        if (cudaStreamIsCapturing(s, &cs) == cudaSuccess && cs == cudaStreamCaptureStatusNone) {
-            const cudaError_t e = rhs_kernels_init();
-            if (e != cudaSuccess) return e;
-            res = rhs_resident<FAM, AX, ORD>();
-        }
-    }
-    const dim3 grd((unsigned)(rhs_strided<AX>() && res > 0 && res < nb ? res : nb));
-    k_rhs<FAM, AX, ORD><<<grd, dim3(RHS_BX, RHS_BY), 0, s>>>(G, yin, d1x, d1y, out, yn, acc, st, oa);
     return cudaGetLastError();
 }
 
@@ -393,37 +369,12 @@ cudaError_t launch_rhs_ord(const GridK& G, const double* yin, double* d1x, doubl
         cudaError_t e = cudaGetLastError();
         if (e != cudaSuccess) return e;
     }
-    oa.nblocks = (oa.npts + RHS_BX * RHS_BY - 1) / (RHS_BX * RHS_BY);
-    const long nb = (long)((G.N0 + RHS_BX - 1) / RHS_BX) * ((G.N1 * G.N2 + RHS_BY - 1) / RHS_BY) + oa.nblocks;
     if (G.fam == FAM_SPH) {
-        if (G.ax == 2) return launch_k_rhs<FAM_SPH, 2, ORD>(nb, s, G, yin, d1x, d1y, out, yn, acc, st, oa);
-        return launch_k_rhs<FAM_SPH, -1, ORD>(nb, s, G, yin, d1x, d1y, out, yn, acc, st, oa);
+        if (G.ax == 2) return launch_k_rhs<FAM_SPH, 2, ORD>(s, G, yin, d1x, d1y, out, yn, acc, st, oa);
+        return launch_k_rhs<FAM_SPH, -1, ORD>(s, G, yin, d1x, d1y, out, yn, acc, st, oa);
     }
-    if (G.ax == 1) return launch_k_rhs<FAM_CYL, 1, ORD>(nb, s, G, yin, d1x, d1y, out, yn, acc, st, oa);
-    return launch_k_rhs<FAM_CYL, -1, ORD>(nb, s, G, yin, d1x, d1y, out, yn, acc, st, oa);
-}
-
-// the resident-block table of every k_rhs instantiation on the current device (idempotent; not
-// during a stream capture)
-cudaError_t rhs_kernels_init()
-{
-    int dev = 0, nsm = 0;
-    cudaError_t e = cudaGetDevice(&dev);
-    if (e != cudaSuccess) return e;
-    if (dev < 0 || dev >= RHS_MAX_DEV) return cudaSuccess;   // launches there run one block per tile
-    std::lock_guard<std::mutex> lk(g_rhs_mu);
-    bool known = true;
-    for (int v = 0; v < RHS_VARIANTS; v++) known = known && g_rhs_resident[dev][v].load() > 0;
-    if (known) return cudaSuccess;
-    if ((e = cudaDeviceGetAttribute(&nsm, cudaDevAttrMultiProcessorCount, dev)) != cudaSuccess) return e;
-    if ((e = rhs_init_one<FAM_SPH, 2, 4>(dev, nsm)) != cudaSuccess) return e;
-    if ((e = rhs_init_one<FAM_SPH, -1, 4>(dev, nsm)) != cudaSuccess) return e;
-    if ((e = rhs_init_one<FAM_CYL, 1, 4>(dev, nsm)) != cudaSuccess) return e;
-    if ((e = rhs_init_one<FAM_CYL, -1, 4>(dev, nsm)) != cudaSuccess) return e;
-    if ((e = rhs_init_one<FAM_SPH, 2, 8>(dev, nsm)) != cudaSuccess) return e;
-    if ((e = rhs_init_one<FAM_SPH, -1, 8>(dev, nsm)) != cudaSuccess) return e;
-    if ((e = rhs_init_one<FAM_CYL, 1, 8>(dev, nsm)) != cudaSuccess) return e;
-    return rhs_init_one<FAM_CYL, -1, 8>(dev, nsm);
+    if (G.ax == 1) return launch_k_rhs<FAM_CYL, 1, ORD>(s, G, yin, d1x, d1y, out, yn, acc, st, oa);
+    return launch_k_rhs<FAM_CYL, -1, ORD>(s, G, yin, d1x, d1y, out, yn, acc, st, oa);
 }
 
 cudaError_t launch_rhs(const GridK& G, const double* yin, double* d1x, double* d1y, double* out, const double* yn,

@@ -164,18 +164,14 @@ __device__ __forceinline__ int gf_type(int g)
     return g - G_BET + 1;
 }
 
-// one interior point (interior-relative i in [0,N0), j = i1 + N1 i2 in [0, N1 N2)) of an RK stage:
-// right-hand side, upwinded advection, dissipation and the stage epilogue.  AX: the azimuthal axis
-// when it holds two points (G.ax), else -1.  S: the raw first differences along axes 0 and 1 of the
-// gridfunctions with second derivatives are read from d1x, d1y (N_D1 sets of T doubles; d1y only
-// for AX = -1), as k_d1 stored them from yin; the result is bitwise the same either way.
-template <int FAM, int AX, bool S, int ORD>
-__device__ __forceinline__ void rhs_point_stage(const GridK& G, const double* __restrict__ yin,
-                                                const double* __restrict__ d1x, const double* __restrict__ d1y,
-                                                double* out, const double* yn, double* acc, const Stage& st, int i,
-                                                int j)
+// the inputs of the point at padded indices p0, p1, p2 but its geometry; d1x, d1y: the raw first differences along
+// axes 0 and 1 of the gridfunctions with second derivatives (N_D1 sets of T doubles; d1y only for AX = -1), as
+// k_d1 stored them from yin.  AX: the azimuthal axis when it holds two points (G.ax), else -1.
+template <int AX>
+__device__ __forceinline__ PointIn point_in(const GridK& G, const double* __restrict__ yin,
+                                            const double* __restrict__ d1x, const double* __restrict__ d1y, int p0,
+                                            int p1, int p2)
 {
-    const int p0 = i + G.NG, p1 = j % G.N1 + G.NG, p2 = j / G.N1 + G.NG;
     const long idx = p0 + (long)G.n0 * (p1 + (long)G.n1 * p2);
     PointIn P;
     P.y = yin + idx;
@@ -186,13 +182,62 @@ __device__ __forceinline__ void rhs_point_stage(const GridK& G, const double* __
     if constexpr (AX == 1) P.ox = p1 == G.NG ? P.st[1] : -P.st[1];
     else if constexpr (AX == 2) P.ox = p2 == G.NG ? P.st[2] : -P.st[2];
     else P.ox = 0;
-    P.dx = S ? d1x + idx : nullptr;
-    P.dy = (S && AX < 0) ? d1y + idx : nullptr;
+    P.dx = d1x + idx;
+    P.dy = AX < 0 ? d1y + idx : nullptr;
+    P.raw = nullptr;
+    return P;
+}
+
+// one interior point (interior-relative i in [0,N0), j = i1 + N1 i2 in [0, N1 N2)) of an RK stage:
+// right-hand side, upwinded advection, dissipation and the stage epilogue.
+template <int FAM, int AX, int ORD>
+__device__ __forceinline__ void rhs_point_stage(const GridK& G, const double* __restrict__ yin,
+                                                const double* __restrict__ d1x, const double* __restrict__ d1y,
+                                                double* out, const double* yn, double* acc, const Stage& st, int i,
+                                                int j)
+{
+    const int p0 = i + G.NG, p1 = j % G.N1 + G.NG, p2 = j / G.N1 + G.NG;
+    PointIn P = point_in<AX>(G, yin, d1x, d1y, p0, p1, p2);
+    // the integer-pipe passes first: their results wait in local memory, the FP64 part needs every register
+    double raw[RawIx<AX>::N], adv[NGF], k[NGF];
+    raw_table<AX, ORD>(P.y, P.dx, P.dy, G.T, P.st, P.ox, raw);
+    P.raw = raw;
+    make_geo_scales<FAM>(G, p0, p1, p2, P.g.D);
+    adv_ko_sums<AX, ORD>(P.y, G.T, P.st, P.ox, P.g.D, G.sigma_metric, G.sigma_gauge, adv);
     P.g = make_geo<FAM>(G, p0, p1, p2);
+    rhs_core<FAM, AX, SRC_TABLE, ORD>(P, G.eta, k);
+#pragma unroll
+    for (int g = 0; g < NGF; g++) k[g] += adv[g];
+    stage_store<ssp_first_short<AX>()>(st, G.T, P.y - yin, k, yin, yn, out, acc);
+}
+
+// 32 interior points (point, lane by lane; lanes without one pass any valid point and active = false) by the
+// SPREAD_WARPS warps of a block: the integer-pipe passes are divided among the warps, then one warp goes on
+// with the FP64 part.  The same arithmetic as rhs_point_stage.  tab: shared memory.
+constexpr int SPREAD_WARPS = 4;
+template <int FAM, int AX, int ORD>
+__device__ __forceinline__ void rhs_spread_stage(const GridK& G, const double* __restrict__ yin,
+                                                 const double* __restrict__ d1x, const double* __restrict__ d1y,
+                                                 double* out, const double* yn, double* acc, const Stage& st, int i,
+                                                 int j, bool active, int warp, int fp_warp,
+                                                 double (*tab)[32])
+{
+    const int lane = threadIdx.x & 31;
+    const int p0 = i + G.NG, p1 = j % G.N1 + G.NG, p2 = j / G.N1 + G.NG;
+    PointIn P = point_in<AX>(G, yin, d1x, d1y, p0, p1, p2);
+    raw_table<AX, ORD>(P.y, P.dx, P.dy, G.T, P.st, P.ox, &tab[0][lane], 32, warp, SPREAD_WARPS);
+    make_geo_scales<FAM>(G, p0, p1, p2, P.g.D);
+    adv_ko_sums<AX, ORD>(P.y, G.T, P.st, P.ox, P.g.D, G.sigma_metric, G.sigma_gauge, &tab[RawIx<AX>::N][lane], 32,
+                         warp, SPREAD_WARPS);
+    __syncthreads();
+    if (warp != fp_warp || !active) return;
     double k[NGF];
-    rhs_core<FAM, AX, S, ORD>(P, G.eta, k);
-    add_adv_ko<AX, ORD>(P.y, G.T, P.st, P.ox, P.g.D, G.sigma_metric, G.sigma_gauge, k);
-    stage_store<ssp_first_short<AX>()>(st, G.T, idx, k, yin, yn, out, acc);
+    P.raw = &tab[0][lane];
+    P.g = make_geo<FAM>(G, p0, p1, p2);
+    rhs_core<FAM, AX, SRC_SHARED, ORD>(P, G.eta, k);
+#pragma unroll
+    for (int g = 0; g < NGF; g++) k[g] += tab[RawIx<AX>::N + g][lane];
+    stage_store<ssp_first_short<AX>()>(st, G.T, P.y - yin, k, yin, yn, out, acc);
 }
 
 // Points of the stored first differences (k_d1): interior i0, and i1 and i2 within

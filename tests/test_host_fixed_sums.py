@@ -1,0 +1,168 @@
+"""The difference sums on the integer pipe (csrc/fixed_sum.cuh), compiled for the host, against rational
+arithmetic.
+
+A first difference is off by less than half an ulp of the result (one rounding) plus one unit of the alignment,
+2^-(52 + SH) of the largest value, for each value and unit of weight.  The advection + dissipation sum is off by
+the same, for u U + kap K summed over the axes, plus the alignment of u and kap to their largest (2^-(52 + 6) of it,
+times the differences), plus what its integers drop at the end: at most 2^-52 (4th order) and 6 x 2^-48 + 2^-46 (8th)
+of the largest coefficient times the largest value.  Sums that the integers cannot hold (infinities, NaNs, values near
+the ends of the exponent range) are the FP64 sums bit for bit.
+"""
+import ctypes
+import os
+import shutil
+import subprocess
+from fractions import Fraction as Fr
+
+import numpy as np
+import pytest
+
+HERE = os.path.dirname(os.path.abspath(__file__))
+D1 = {4: {-2: 1, -1: -8, 1: 8, 2: -1}, 8: {-4: 3, -3: -32, -2: 168, -1: -672, 1: 672, 2: -168, 3: 32, 4: -3}}
+UP = {4: {-1: -3, 0: -10, 1: 18, 2: -6, 3: 1},
+      8: {-3: -5, -2: 60, -1: -420, 0: -378, 1: 1050, 2: -420, 3: 140, 4: -30, 5: 3}}
+KO = {4: (1, -6, 15, -20, 15, -6, 1), 8: (1, -10, 45, -120, 210, -252, 210, -120, 45, -10, 1)}
+KC = {4: Fr(12, 64), 8: Fr(840, 1024)}
+dp = ctypes.POINTER(ctypes.c_double)
+
+
+def _p(a):
+    return a.ctypes.data_as(dp)
+
+
+@pytest.fixture(scope="module")
+def lib(tmp_path_factory):
+    gxx = shutil.which("g++")
+    if gxx is None:
+        pytest.skip("g++ not found")
+    so = str(tmp_path_factory.mktemp("fixed") / "fixed.so")
+    r = subprocess.run([gxx, "-O2", "-std=c++17", "-shared", "-fPIC", "-ffp-contract=off", "-Wno-unknown-pragmas",
+                        os.path.join(HERE, "host_point", "fixed_point.cpp"), "-o", so], capture_output=True, text=True)
+    assert r.returncode == 0, r.stderr
+    return ctypes.CDLL(so)
+
+
+def _rows(rng, kind, n, width):
+    if kind == "smooth":
+        x = np.linspace(0, 1, width)[None, :]
+        a, k, p = rng.uniform(-1, 1, (3, n, 1))
+        return (a + 1e-3 * np.cos(3 * k * x + 6 * p)) * 10.0 ** rng.uniform(-12, 3, (n, 1))
+    if kind == "binades":      # exponents far apart, both signs, zeros of both signs among them
+        f = rng.uniform(-1, 1, (n, width)) * 2.0 ** rng.integers(-80, 3, (n, width))
+        f[rng.uniform(size=f.shape) < 0.1] = 0.0
+        f[rng.uniform(size=f.shape) < 0.05] = -0.0
+        return f
+    return rng.uniform(-1, 1, (n, width))
+
+
+@pytest.mark.parametrize("kind", ["smooth", "noise", "binades"])
+@pytest.mark.parametrize("order", [4, 8])
+def test_first_difference(lib, order, kind):
+    rng = np.random.default_rng(order)
+    f = np.ascontiguousarray(_rows(rng, kind, 400, 9))
+    out, fp = np.empty(len(f)), np.empty(len(f))
+    lib.fixed_d1(order, _p(f), ctypes.c_long(len(f)), _p(out), _p(fp))
+    sh = 5 if order == 4 else 9
+    weight = sum(abs(w) for w in D1[order].values())
+    worse = 0
+    for row, o, g in zip(f, out, fp):
+        exact = sum(w * Fr(row[4 + j]) for j, w in D1[order].items())
+        big = max(abs(Fr(row[4 + j])) for j in D1[order])
+        assert abs(Fr(o) - exact) <= abs(exact) / 2 ** 53 + weight * big / 2 ** (52 + sh)
+        worse += abs(Fr(o) - exact) - abs(Fr(g) - exact)
+    assert worse <= 0          # summed over the rows, no further off than the FP64 sums
+
+
+@pytest.mark.parametrize("bad", [np.inf, -np.inf, np.nan, 1e308, 1e-290, 5e-324])
+@pytest.mark.parametrize("order", [4, 8])
+def test_first_difference_outside_the_range_is_the_fp64_sum(lib, order, bad):
+    f = np.full((1, 9), bad) if abs(bad) < 1e-200 else np.random.default_rng(1).uniform(-1, 1, (1, 9))
+    f[0, 2] = bad
+    f[0, 5] *= 0.5
+    out, fp = np.empty(1), np.empty(1)
+    lib.fixed_d1(order, _p(f), ctypes.c_long(1), _p(out), _p(fp))
+    assert np.array_equal(out, fp, equal_nan=True)
+
+
+def test_subtraction_is_the_ieee_difference_of_neighbours(lib):
+    rng = np.random.default_rng(3)
+    a = rng.uniform(-1, 1, 5000) * 2.0 ** rng.integers(-200, 200, 5000)
+    b = a * rng.choice([1.0, 1.0 + 1e-9, 0.7, -1.0, 1.3, 0.0], 5000)
+    a[:3], b[:3] = (0.0, np.inf, 1e300), (0.0, 1.0, -1e300)
+    out = np.empty(5000)
+    lib.fixed_sub(_p(a), _p(b), ctypes.c_long(5000), _p(out))
+    near = np.abs(a - b) <= np.maximum(np.abs(a), np.abs(b)) / 2   # exact in FP64
+    with np.errstate(invalid="ignore"):
+        assert np.array_equal(out[near], (a - b)[near])
+        assert np.all(np.abs(out[3:] - (a - b)[3:]) <= 2.0 ** -52 * np.maximum(np.abs(a), np.abs(b))[3:])
+    assert out[0] == 0.0 and out[1] == np.inf and out[2] == 2e300 - 0.0
+
+
+def _exact_advko(order, ax, f, vet, D, sigma):
+    n = 11
+    at = lambda d, o: Fr(float(f[tuple(5 + (o if 2 - i == d else 0) for i in range(3))]))  # noqa: E731
+    G = len(KO[order]) // 2
+    tot = Fr(0)
+    for d in range(3):
+        u = abs(Fr(float(abs(vet[d]) * D[d])))
+        kap = Fr(float(float(KC[order]) * sigma * D[d]))
+        if d == ax:
+            tot += ({4: 16, 8: 768}[order] * u + {4: 32, 8: 512}[order] * kap) * (at(d, 1) - at(d, 0))
+            continue
+        s = 1 if vet[d] > 0 else -1
+        tot += u * sum(w * at(d, s * o) for o, w in UP[order].items())
+        tot += kap * sum(w * at(d, o - G) for o, w in enumerate(KO[order]))
+    assert n == f.shape[0]
+    return tot
+
+
+@pytest.mark.parametrize("kind", ["smooth", "noise", "binades"])
+@pytest.mark.parametrize("ax", [-1, 1, 2])
+@pytest.mark.parametrize("order", [4, 8])
+def test_advection_and_dissipation(lib, order, ax, kind):
+    rng = np.random.default_rng(10 * order + ax)
+    up, ko = sum(abs(w) for w in UP[order].values()), sum(abs(w) for w in KO[order])
+    sh = 2 if order == 4 else 5
+    worse = 0
+    for _ in range(40):
+        f = np.ascontiguousarray(_rows(rng, kind, 1, 11 ** 3).reshape(11, 11, 11))
+        vet = rng.uniform(-0.3, 0.3, 3) * 10.0 ** rng.uniform(-8, 0, 3) * (rng.uniform(size=3) > 0.15)
+        D = 10.0 ** rng.uniform(-3, 3, 3)
+        sigma = float(rng.choice([0.3, 0.99, 1e-6]))
+        out, fp = np.empty(1), np.empty(1)
+        lib.fixed_advko(ax, order, _p(f), _p(vet), _p(D), ctypes.c_double(sigma), _p(out), _p(fp))
+        exact = _exact_advko(order, ax, f, vet, D, sigma)
+        c = max([abs(Fr(float(abs(v) * d))) for v, d in zip(vet, D)] + [Fr(float(float(KC[order]) * sigma * d)) for d in D])
+        axes = [f[tuple(slice(None) if 2 - i == d else 5 for i in range(3))] for d in range(3) if d != ax]
+        vals = np.concatenate(axes + ([f[tuple(6 if 2 - i == ax else 5 for i in range(3))].reshape(1)] if ax >= 0 else []))
+        big = Fr(float(np.abs(vals).max()))
+        weights = 3 * (up + ko) + (2 * (768 + 512) if order == 8 else 2 * 48)
+        last = Fr(1, 2 ** 52) if order == 4 else Fr(6, 2 ** 48) + Fr(1, 2 ** 46)
+        bound = abs(exact) / 2 ** 53 + c * big * (weights * (Fr(1, 2 ** (52 + sh)) + Fr(1, 2 ** 58)) + last)
+        assert abs(Fr(float(out[0])) - exact) <= bound
+        worse += (abs(Fr(float(out[0])) - exact) - abs(Fr(float(fp[0])) - exact)) / (c * big) if big else 0
+    # summed over the draws, no further off than the FP64 sum; not claimed for values scattered over 80 binades, whose
+    # FP64 sum is often one product: there the alignment's 2^-(52 + SH) of the largest value is the larger error
+    # (up to 6 times, at 4e-17 of the largest product)
+    assert kind == "binades" or worse <= 0
+
+
+@pytest.mark.parametrize("bad", [np.inf, np.nan, 1e306, 5e-324])
+@pytest.mark.parametrize("where", ["value", "shift"])
+@pytest.mark.parametrize("order", [4, 8])
+def test_advection_outside_the_range_is_the_fp64_sum(lib, order, where, bad):
+    rng = np.random.default_rng(5)
+    f = np.ascontiguousarray(rng.uniform(-1, 1, (11, 11, 11)))
+    vet, D = np.array([0.1, -0.2, 0.05]), np.array([3.0, 1.0, 2.0])
+    if where == "shift":
+        vet[1] = bad
+        if abs(bad) < 1:       # an underflowing advection speed beside ordinary ones is no special case
+            vet[:] = bad
+            D[:] = 1e-310
+    elif abs(bad) < 1:
+        f *= bad
+    else:
+        f[5, 5, 7] = bad
+    out, fp = np.empty(1), np.empty(1)
+    lib.fixed_advko(-1, order, _p(f), _p(vet), _p(D), ctypes.c_double(0.3), _p(out), _p(fp))
+    assert np.array_equal(out, fp, equal_nan=True)
