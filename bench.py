@@ -56,7 +56,7 @@ UNIT = "point-updates/s"
 # as the point code's source has them (add + mul + div + 2 fma, a host census that a test recomputes), with
 # the raw first differences counted as FP64 sums.  The kernels take those, and the advection + dissipation sums
 # (not counted here at all), in integer arithmetic beside the FP64 pipe.
-F_ALG = {"headon": 2294.3, "large3d": 3306.8, "headon8": 2736.9, "large3d8": 4092.2}
+F_ALG = {"headon": 2051.3, "large3d": 2933.8, "headon8": 2493.9, "large3d8": 3719.2}
 # DRAM bytes (read + write) of the same two launches in that capture; for the large 3D grids the
 # capture's bytes per interior point at 96x48x96 (3275.7 and 5324.5, mostly register-spill lines)
 # times the 28,311,552 points of the full grid
@@ -64,10 +64,10 @@ TRAFFIC = {"headon": 24016384 + 88832 + 94202624 + 510593792,
            "headon8": 24951296 + 119552 + 94502400 + 486498304,
            "large3d": round(3275.7 * 28311552), "large3d8": round(5324.5 * 28311552)}
 # The same without the k_d1 pre-pass
-KERNEL_CENSUS = {"headon": 2250, "headon8": 2614, "large3d": 3217, "large3d8": 3840}
+KERNEL_CENSUS = {"headon": 2007, "headon8": 2371, "large3d": 2844, "large3d8": 3467}
 # FLOPs over twice the FP64 instructions of the same source (k_d1 + k_rhs): the fraction of the FLOP peak
 # that a fully busy FP64 pipe reaches with this mix (a DADD or DMUL takes an FMA's issue slot for 1 FLOP)
-MIX_CEILING = {"headon": 0.7932, "headon8": 0.7765, "large3d": 0.8005, "large3d8": 0.7790}
+MIX_CEILING = {"headon": 0.7810, "headon8": 0.7653, "large3d": 0.7906, "large3d8": 0.7696}
 # FP64 operations (add + mul + div) per interior point of one RHS evaluation as the oracle's counting
 # build counts them: the plain coordinate-basis evaluation of the same discretisation with generic index
 # loops and the reference metric evaluated at every point -- the work of the method evaluated plainly.
@@ -76,12 +76,12 @@ MIX_CEILING = {"headon": 0.7932, "headon8": 0.7765, "large3d": 0.8005, "large3d8
 F_METHOD = {"headon": 28967, "headon8": 49631, "large3d": 28970, "large3d8": 49634}
 # The same for the diagnostics (Hamiltonian and momentum constraints, psi4), per interior
 # point of one call, from one ncu capture of those kernels on the head-on state, by workload
-# (head-on: k_ham 366 / 238 / 640 DADD / DMUL / DFMA, k_mom 119 / 162 / 269, k_psi4 505 / 483 /
-# 1085; the reductions and ghost copies add < 0.1); absent: not captured
-DIAG_FLOPS = {"headon": {"hamiltonian": 1884.0, "momentum": 819.0, "psi4": 3158.0}}
+# (head-on: k_ham 363 / 218 / 593 DADD / DMUL / DFMA, k_mom 111 / 142 / 262, k_psi4 460 / 434 /
+# 1016; the reductions and ghost copies add < 0.1); absent: not captured
+DIAG_FLOPS = {"headon": {"hamiltonian": 1767.0, "momentum": 777.0, "psi4": 2926.0}}
 # the source census of the constraints' point code those counts were taken with (FMA = 2, one division,
-# the square root of |M| not counted: its expansion is most of the 29 FLOP the momentum count adds)
-DIAG_CENSUS = {"headon": {"hamiltonian": 1881, "momentum": 785}}
+# the square root of |M| not counted: its expansion is most of the 34 FLOP the momentum count adds)
+DIAG_CENSUS = {"headon": {"hamiltonian": 1773, "momentum": 743}}
 # psi4 modes on the workload's extraction sphere: l <= 8, Gauss-Legendre x uniform nodes
 PSI4_LMAX, PSI4_NTHETA, PSI4_NPHI = 8, 24, 48
 # FP64 pipe of one SM: 2 DFMA per clock (ncu peak_sustained of

@@ -202,6 +202,12 @@ __host__ __device__ constexpr bool dlz(int k, int s)
 {
     return FAM == FAM_CYL && AX == 1 && k == 2 && s == 4;
 }
+// Dhat_k h_ij (s = ij) known to vanish: Omega_1 h leaves the (2,2) component alone
+template <int FAM, int AX>
+__host__ __device__ constexpr bool dhz(int k, int s)
+{
+    return FAM == FAM_CYL && AX == 1 && k == 1 && s == 5;
+}
 // Dhat_k Dhat_l V^i known to vanish (kl symmetric index): on a cylindrical-like grid
 // with a two-point azimuth, the (rho, phi) and (phi, z) pairs of component z
 template <int FAM, int AX>
@@ -431,13 +437,15 @@ struct MetricPart {
     double h[6], gi[6], gw[6];
     double dh[3][6];
     double GH[6];        // gammabar^ij H_kl h_ij
-    double Dl[3][6];     // Delta_kij (first index lowered)
+    double Dh[3][6];     // Dhat_k h_ij
+    double Dl2[3][6];    // 2 Delta_kij (first index lowered)
     double Dup[3][6];    // Delta^k_ij
     double Dvec[3];      // Delta^k
     double Dtr[3];       // Delta^k_km
     double Ric[6];       // Rbar_ij
     double W, iW, dphi[3];
-    double DDphir[6];    // Dbar_i Dbar_j phi - 2 e_i phi e_j phi (what every consumer needs)
+    double HW[6];        // H_ij W (right-hand side)
+    double DDphir[6];    // Dbar_i Dbar_j phi - 2 e_i phi e_j phi (the diagnostics)
 };
 
 // The conformal metric and its inverse, first frame derivatives of h, and
@@ -484,33 +492,36 @@ __device__ __forceinline__ void metric_first(const PointIn& P, MetricPart& M)
         for (int s = 0; s < 6; s++) dh[k][s] = der1<AX, S, ORD>(P, G_HDD + s, k);
 
     // ---------------- Dhat_k h_ij, Delta_kij (first index lowered), Delta^k_ij, Delta^k
-    double Dh[3][6];
+    double (*Dh)[6] = M.Dh;
 #pragma unroll
     for (int s = 0; s < 6; s++) { Dh[0][s] = dh[0][s]; Dh[1][s] = dh[1][s]; Dh[2][s] = dh[2][s]; }
     oms<FAM, 1>(g, h, Dh[1]);
     oms<FAM, 2>(g, h, Dh[2]);
-    double (*Dl)[6] = M.Dl;
+    // 2 Delta_kij = Dhat_i h_jk + Dhat_j h_ik - Dhat_k h_ij; with k = j (k = i) the last two (the first and
+    // last) terms are the same number and cancel exactly.  The 1/2 goes into gammabar^kl / 2.
+    double (*Dl2)[6] = M.Dl2;
 #pragma unroll
     for (int k = 0; k < 3; k++)
 #pragma unroll
         for (int s = 0; s < 6; s++) {
             const int i = spi(s), j = spj(s);
-            // Delta_kij = 1/2 (Dhat_i h_jk + Dhat_j h_ik - Dhat_k h_ij); with k = j (k = i) the
-            // last two (the first and last) terms are the same number and cancel exactly
             if (k == j)
-                Dl[k][s] = sc2<-1>(Dh[i][sp(k, k)]);
+                Dl2[k][s] = Dh[i][sp(k, k)];
             else if (k == i)
-                Dl[k][s] = sc2<-1>(Dh[j][sp(k, k)]);
+                Dl2[k][s] = Dh[j][sp(k, k)];
             else
-                Dl[k][s] = sc2<-1>(Dh[i][sp(j, k)] + Dh[j][sp(i, k)] - Dh[k][s]);
+                Dl2[k][s] = Dh[i][sp(j, k)] + Dh[j][sp(i, k)] - Dh[k][s];
         }
+    double gh[6];   // gammabar^kl / 2
+#pragma unroll
+    for (int s = 0; s < 6; s++) gh[s] = sc2<-1>(gi[s]);
     double (*Dup)[6] = M.Dup;
 #pragma unroll
     for (int k = 0; k < 3; k++)
 #pragma unroll
         for (int s = 0; s < 6; s++) {
-            double t = fma(gsym(gi, k, 1), Dl[1][s], gsym(gi, k, 0) * Dl[0][s]);
-            Dup[k][s] = dlz<FAM, AX>(2, s) ? t : fma(gsym(gi, k, 2), Dl[2][s], t);
+            double t = fma(gsym(gh, k, 1), Dl2[1][s], gsym(gh, k, 0) * Dl2[0][s]);
+            Dup[k][s] = dlz<FAM, AX>(2, s) ? t : fma(gsym(gh, k, 2), Dl2[2][s], t);
         }
     double* Dvec = M.Dvec;
 #pragma unroll
@@ -520,14 +531,9 @@ __device__ __forceinline__ void metric_first(const PointIn& P, MetricPart& M)
         for (int s = 1; s < 6; s++) t = fma(gw[s], Dup[k][s], t);
         Dvec[k] = t;
     }
-    // Delta^k_km = 1/2 gammabar^ab e_m h_ab
+    // Delta^k_km (= 1/2 gammabar^ab e_m h_ab: zero along the two-point axis)
 #pragma unroll
-    for (int m = 0; m < 3; m++) {
-        double t = gw[0] * dh[m][0];
-#pragma unroll
-        for (int s = 1; s < 6; s++) t = fma(gw[s], dh[m][s], t);
-        M.Dtr[m] = m == AX ? 0.0 : sc2<-1>(t);
-    }
+    for (int m = 0; m < 3; m++) M.Dtr[m] = m == AX ? 0.0 : Dup[0][sp(0, m)] + Dup[1][sp(1, m)] + Dup[2][sp(2, m)];
 }
 
 template <int FAM, bool NEED_GH, int AX, int S, int ORD>
@@ -543,7 +549,8 @@ __device__ __forceinline__ void metric_part(const PointIn& P, MetricPart& M)
     const double* gi = M.gi;
     const double* gw = M.gw;
     const double (*dh)[6] = M.dh;
-    const double (*Dl)[6] = M.Dl;
+    const double (*Dh)[6] = M.Dh;
+    const double (*Dl2)[6] = M.Dl2;
     const double (*Dup)[6] = M.Dup;
     const double* Dvec = M.Dvec;
 
@@ -619,11 +626,14 @@ __device__ __forceinline__ void metric_part(const PointIn& P, MetricPart& M)
     omv<FAM, 1>(g, lam, Dlam[1]);
     omv<FAM, 2>(g, lam, Dlam[2]);
     // Quadratic terms. With R[i][m][l] = gammabar^lk Delta^m_ik,
-    //   gammabar^kl Delta^m_ki Delta_jml = sum_ml R[i][m][l] Delta_jml   (A_ij; Delta_jml is
-    //                                      symmetric in ml, so R is summed over the pair first)
-    //   gammabar^kl Delta^m_ik Delta_mjl = sum_ml R[i][m][l] Delta_mjl   (C_ij, symmetric)
-    // and R_ij = -1/2 Lfull_ij + A_ij + A_ji + C_ij + 1/2 (Lambda and Delta^k terms), each
-    // component one chain with the 1/2 taken into the factors.
+    //   A_ij = gammabar^kl Delta^m_ki Delta_jml = sum_ml R[i][m][l] Delta_jml
+    //   C_ij = gammabar^kl Delta^m_ik Delta_mjl = sum_ml R[i][m][l] Delta_mjl   (symmetric)
+    // and Delta_jml + Delta_mjl = Dhat_l h_jm, so
+    //   A_ij + A_ji + C_ij = sum_ml R[i][m][l] Dhat_l h_jm + sum_ml R[j][m][l] Delta_iml,
+    // the last sum over R's pair sums (Delta_iml is symmetric in ml).  R_ij = -1/2 Lfull_ij + A_ij + A_ji + C_ij
+    // + 1/2 (Lambda and Delta^k terms), in which Delta^k (Delta_ijk + Delta_jik) = Delta^k Dhat_k h_ij: each
+    // component is one chain of the terms without the 1/2 and one of those with it, halved by the FMA that
+    // adds it.
     double R[3][3][3];
 #pragma unroll
     for (int i = 0; i < 3; i++)
@@ -641,47 +651,29 @@ __device__ __forceinline__ void metric_part(const PointIn& P, MetricPart& M)
 #pragma unroll
     for (int s = 0; s < 6; s++) {
         const int i = spi(s), j = spj(s);
-        // C_ij
-        double t = R[i][0][0] * Dl[0][sp(j, 0)];
+        double t = R[i][0][0] * Dh[0][sp(j, 0)];
 #pragma unroll
         for (int q = 1; q < 9; q++) {
             const int m = q / 3, l = q % 3;
-            if (!dlz<FAM, AX>(m, sp(j, l))) t = fma(R[i][m][l], Dl[m][sp(j, l)], t);
+            if (!dhz<FAM, AX>(l, sp(j, m))) t = fma(R[i][m][l], Dh[l][sp(j, m)], t);
         }
-        // (Dl[k][p] = 0 where dlz(k, p) and Dlam[j][k] = Dhat_j lambda^k = 0 where dvz(k, j):
+        // (Dl2[k][p] = 0 where dlz(k, p) and Dlam[j][k] = Dhat_j lambda^k = 0 where dvz(k, j):
         // those terms are skipped)
+        double v = -Lfull[s];
+#pragma unroll
+        for (int p = 0; p < 6; p++)
+            if (!dlz<FAM, AX>(i, p)) v = fma(Rp[j][p], Dl2[i][p], v);
+#pragma unroll
+        for (int k = 0; k < 3; k++)
+            if (!dhz<FAM, AX>(k, s)) v = fma(Dvec[k], Dh[k][s], v);
         if (i == j) {
-            // 2 A_ii (A_ii summed on its own, doubled by the FMA that adds it)
-            double u = 0.0;
-#pragma unroll
-            for (int p = 0; p < 6; p++)
-                if (!dlz<FAM, AX>(i, p)) u = fma(Rp[i][p], Dl[i][p], u);
-            t = fma(2.0, u, t);
-            // 1/2 Delta^k (2 Delta_iik)
-#pragma unroll
-            for (int k = 0; k < 3; k++)
-                if (!dlz<FAM, AX>(i, sp(i, k))) t = fma(Dvec[k], Dl[i][sp(i, k)], t);
             // 1/2 (2 gammabar_ki Dhat_i lambda^k)
             if (!dvz<FAM, AX>(i, i)) t += Dlam[i][i];
 #pragma unroll
             for (int k = 0; k < 3; k++)
                 if (!dvz<FAM, AX>(k, i)) t = fma(h[sp(k, i)], Dlam[i][k], t);
         } else {
-            // A_ij + A_ji
-#pragma unroll
-            for (int p = 0; p < 6; p++)
-                if (!dlz<FAM, AX>(j, p)) t = fma(Rp[i][p], Dl[j][p], t);
-#pragma unroll
-            for (int p = 0; p < 6; p++)
-                if (!dlz<FAM, AX>(i, p)) t = fma(Rp[j][p], Dl[i][p], t);
-            // 1/2 Delta^k (Delta_ijk + Delta_jik) + 1/2 (gammabar_ki Dhat_j lambda^k + gammabar_kj
-            // Dhat_i lambda^k): summed on their own, halved by the FMA that adds them
-            double v = 0.0;
-#pragma unroll
-            for (int k = 0; k < 3; k++) {
-                if (!dlz<FAM, AX>(i, sp(j, k))) v = fma(Dvec[k], Dl[i][sp(j, k)], v);
-                if (!dlz<FAM, AX>(j, sp(i, k))) v = fma(Dvec[k], Dl[j][sp(i, k)], v);
-            }
+            // gammabar_ki Dhat_j lambda^k + gammabar_kj Dhat_i lambda^k
             if (!dvz<FAM, AX>(i, j)) v += Dlam[j][i];
             if (!dvz<FAM, AX>(j, i)) v += Dlam[i][j];
 #pragma unroll
@@ -689,9 +681,8 @@ __device__ __forceinline__ void metric_part(const PointIn& P, MetricPart& M)
                 if (!dvz<FAM, AX>(k, i)) v = fma(h[sp(k, j)], Dlam[i][k], v);
                 if (!dvz<FAM, AX>(k, j)) v = fma(h[sp(k, i)], Dlam[j][k], v);
             }
-            t = fma(0.5, v, t);
         }
-        M.Ric[s] = fma(-0.5, Lfull[s], t);
+        M.Ric[s] = fma(0.5, v, t);
     }
 
     // ---------------- conformal factor: phi = -1/2 ln W
@@ -702,8 +693,9 @@ __device__ __forceinline__ void metric_part(const PointIn& P, MetricPart& M)
 #pragma unroll
     for (int k = 0; k < 3; k++) M.dphi[k] = k == AX ? 0.0 : mhiW * dW[k];
     {
-        double HW[6];
+        double* HW = M.HW;
         hess6<FAM, AX, S, ORD>(F(G_CF), dxp<S>(P, G_CF), dyp<AX, S>(P, G_CF), P.raw, d1slot(G_CF), st, P.ox, g, dW, HW);
+        if constexpr (!NEED_GH)
 #pragma unroll
         for (int s = 0; s < 6; s++) {
             // e_i e_j phi = -1/2 W^-1 H_ij W + 2 e_i phi e_j phi; the second term is left out
@@ -735,9 +727,10 @@ __device__ __forceinline__ void rhs_core(const PointIn& P, double eta, double ou
     const double* Dtr = M.Dtr;
     const double* GH = M.GH;
     const double* Ric = M.Ric;
-    const double* dphi = M.dphi;
-    const double* DDphir = M.DDphir;
     const double W = M.W;
+    double dphi2[3];   // 2 e_k phi = -W^-1 e_k W
+#pragma unroll
+    for (int k = 0; k < 3; k++) dphi2[k] = k == AX ? 0.0 : sc2<1>(M.dphi[k]);
 
     double a[6], lam[3], vet[3], bet[3];
 #pragma unroll
@@ -754,16 +747,9 @@ __device__ __forceinline__ void rhs_core(const PointIn& P, double eta, double ou
 #pragma unroll
         for (int i = 0; i < 3; i++) dvet[k][i] = der1<AX, S, ORD>(P, G_VET + i, k);
     }
-    double DDal[6];
-    {
-        double Hal[6];
-        hess6<FAM, AX, S, ORD>(F(G_ALPHA), dxp<S>(P, G_ALPHA), dyp<AX, S>(P, G_ALPHA), P.raw, d1slot(G_ALPHA), st, P.ox, g, dal, Hal);
-#pragma unroll
-        for (int s = 0; s < 6; s++) {
-            const double dd = dot3<AX>(Dup[0][s], Dup[1][s], Dup[2][s], dal);
-            DDal[s] = hzero(AX, s) ? -dd : Hal[s] - dd;
-        }
-    }
+    double Hal[6];
+    hess6<FAM, AX, S, ORD>(F(G_ALPHA), dxp<S>(P, G_ALPHA), dyp<AX, S>(P, G_ALPHA), P.raw, d1slot(G_ALPHA), st, P.ox, g,
+                           dal, Hal);
 
     // ---------------- Abar with raised indices
     double Aud[3][3];  // Abar^k_j
@@ -890,47 +876,50 @@ __device__ __forceinline__ void rhs_core(const PointIn& P, double eta, double ou
     // e_l(Delta^k_km) = 1/2 (GH_lm - Q_lm) - (Omega_l Dtr)_m,  Q_lm = tr(gbinv e_l h gbinv e_m h)
     double gdiv[3];
     {
-        double M[3][3][3];  // M[l] = gbinv . e_l h  (zero along the two-point axis)
-#pragma unroll
-        for (int l = 0; l < 3; l++)
-#pragma unroll
-            for (int i = 0; i < 3; i++)
-#pragma unroll
-                for (int j = 0; j < 3; j++)
-                    M[l][i][j] = l == AX ? 0.0 : fma(gsym(gi, i, 2), dh[l][sp(2, j)], fma(gsym(gi, i, 1), dh[l][sp(1, j)], gsym(gi, i, 0) * dh[l][sp(0, j)]));
-        double Q[6];
+        // sum_m Q_lm vet^m = sum_ab e_l h_ab X^ab with X = gbinv (vet^m e_m h) gbinv
+        double E[6], N[3][3], X[6];
 #pragma unroll
         for (int s = 0; s < 6; s++) {
-            const int l = spi(s), m = spj(s);
-            if (l == AX || m == AX) {
-                Q[s] = 0.0;
-                continue;
-            }
-            double t = M[l][0][0] * M[m][0][0];
-#pragma unroll
-            for (int q = 1; q < 9; q++) t = fma(M[l][q / 3][q % 3], M[m][q % 3][q / 3], t);
-            Q[s] = t;
+            const double d[3] = {dh[0][s], dh[1][s], dh[2][s]};
+            E[s] = dot3<AX>(vet[0], vet[1], vet[2], d);
         }
-        double OD[3][3] = {{0, 0, 0}, {0, 0, 0}, {0, 0, 0}};  // (Omega_l Dtr)
-        omv<FAM, 1>(g, Dtr, OD[1]);
-        omv<FAM, 2>(g, Dtr, OD[2]);
+#pragma unroll
+        for (int i = 0; i < 3; i++)
+#pragma unroll
+            for (int j = 0; j < 3; j++)
+                N[i][j] = fma(gsym(gi, i, 2), E[sp(2, j)], fma(gsym(gi, i, 1), E[sp(1, j)], gsym(gi, i, 0) * E[sp(0, j)]));
+#pragma unroll
+        for (int s = 0; s < 6; s++) {
+            const int i = spi(s), j = spj(s);
+            const double x = fma(N[i][2], gsym(gi, 2, j), fma(N[i][1], gsym(gi, 1, j), N[i][0] * gsym(gi, 0, j)));
+            X[s] = offd(s) ? sc2<1>(x) : x;
+        }
 #pragma unroll
         for (int l = 0; l < 3; l++) {
             double t = DDb[sp(l, 0)][0] + DDb[sp(l, 1)][1];
             if (!ddbz<FAM, AX>(sp(l, 2), 2)) t += DDb[sp(l, 2)][2];
+            // Delta^k_km e_l vet^m - (Omega_l Dtr)_m vet^m = Delta^k_km Dhat_l vet^m
 #pragma unroll
-            for (int m = 0; m < 3; m++) {
-                // with exactly one of l, m on the two-point axis, GH, Q and (Omega_l Dtr)_m all
-                // vanish; Dtr[AX] = 0 and e_AX vet = 0
-                if (l != AX && m != AX) t = fma(Dtr[m], dvet[l][m], t);
-                if (AX < 0 || (l == AX) == (m == AX)) {
-                    const double edtr = fma(0.5, GH[sp(l, m)] - Q[sp(l, m)], -OD[l][m]);
-                    t = fma(edtr, vet[m], t);
-                }
-            }
-            gdiv[l] = t;
+            for (int m = 0; m < 3; m++)
+                if (m != AX && !dvz<FAM, AX>(m, l)) t = fma(Dtr[m], Db[m][l], t);
+            // with exactly one of l, m on the two-point axis, GH vanishes; Q does with either
+            double q = 0.0;
+#pragma unroll
+            for (int m = 0; m < 3; m++)
+                if (AX < 0 || (l == AX) == (m == AX)) q = fma(GH[sp(l, m)], vet[m], q);
+            if (l != AX)
+#pragma unroll
+                for (int s = 0; s < 6; s++) q = fma(-dh[l][s], X[s], q);
+            gdiv[l] = fma(0.5, q, t);
         }
     }
+    // Dhat_j beta^k - alpha Abar^k_j: with gammabar_ik Abar^k_j = a_ij and a_ik Abar^k_j symmetric, it carries the
+    // - 2 alpha a_ij of d_t h and the - 2 alpha a_ik Abar^k_j of d_t a in the terms that hold Dhat_j beta^k
+    double Z[3][3];
+#pragma unroll
+    for (int k = 0; k < 3; k++)
+#pragma unroll
+        for (int j = 0; j < 3; j++) Z[k][j] = dvz<FAM, AX>(k, j) ? -al * Aud[k][j] : fma(-al, Aud[k][j], Db[k][j]);
 
     // ================= right-hand sides (advection and dissipation excluded)
     // Eq. metric_RHS_orig_final + Lie terms:
@@ -938,20 +927,21 @@ __device__ __forceinline__ void rhs_core(const PointIn& P, double eta, double ou
     //            - 2/3 gammabar_ij (Dbar.beta - alpha Abar^k_k) - 2 alpha a_ij
     {
         double r[6];
-        const double tt = (2.0 / 3.0) * fma(-al, trA, divbar);
+        // the trace term as a multiple of the identity in Z, then gammabar Z and its transpose
+        const double t3 = (1.0 / 3.0) * fma(-al, trA, divbar);
+        double Y[3][3];
+#pragma unroll
+        for (int j = 0; j < 3; j++) {
+            const double z[3] = {j == 0 ? Z[0][j] - t3 : Z[0][j], j == 1 ? Z[1][j] - t3 : Z[1][j],
+                                 j == 2 ? Z[2][j] - t3 : Z[2][j]};
+#pragma unroll
+            for (int i = 0; i < 3; i++)
+                Y[i][j] = fma(h[sp(i, 2)], z[2], fma(h[sp(i, 1)], z[1], fma(h[sp(i, 0)], z[0], z[i])));
+        }
 #pragma unroll
         for (int s = 0; s < 6; s++) {
             const int i = spi(s), j = spj(s);
-            // (Db[k][i] = 0 where dvz(k, i): those terms are skipped)
-            const bool zji = dvz<FAM, AX>(j, i), zij = dvz<FAM, AX>(i, j);
-            double t = zji ? (zij ? 0.0 : Db[i][j]) : (zij ? Db[j][i] : Db[j][i] + Db[i][j]);
-#pragma unroll
-            for (int k = 0; k < 3; k++) {
-                if (!dvz<FAM, AX>(k, j)) t = fma(h[sp(i, k)], Db[k][j], t);
-                if (!dvz<FAM, AX>(k, i)) t = fma(h[sp(k, j)], Db[k][i], t);
-            }
-            const double gij = (i == j) ? 1.0 + h[s] : h[s];
-            r[s] = fma(-al2, a[s], fma(-tt, gij, t));
+            r[s] = i == j ? sc2<1>(Y[i][i]) : Y[i][j] + Y[j][i];
         }
         oms<FAM, 1>(g, vet[1], h, r);
         oms<FAM, 2>(g, vet[2], h, r);
@@ -960,17 +950,24 @@ __device__ __forceinline__ void rhs_core(const PointIn& P, double eta, double ou
     }
     // Eq. Abar_RHS_orig_final + Lie terms
     {
-        double X[6];
+        double X[6], dap[3];
+        const double aiW = al * M.iW;
+#pragma unroll
+        for (int k = 0; k < 3; k++) dap[k] = k == AX ? 0.0 : fma(al, dphi2[k], dal[k]);
 #pragma unroll
         for (int s = 0; s < 6; s++) {
             const int i = spi(s), j = spj(s);
-            // 2 alpha (2 e_i phi e_j phi - Dbar_i Dbar_j phi) = -2 alpha DDphir, and
-            // 2 (e_i alpha e_j phi + e_j alpha e_i phi), which vanishes when i or j is the
-            // two-point axis
-            double t = fma(-al2, DDphir[s], -DDal[s]);
+            // -2 alpha (Dbar_i Dbar_j phi - 2 e_i phi e_j phi) - Dbar_i Dbar_j alpha =
+            //   alpha W^-1 H_ij W - H_ij alpha + Delta^k_ij (2 alpha e_k phi + e_k alpha),
+            // and 2 (e_i alpha e_j phi + e_j alpha e_i phi), which vanishes when i or j is the two-point axis
+            double t;
+            if (hzero(AX, s)) t = Dup[0][s] * dap[0];
+            else t = fma(Dup[0][s], dap[0], fma(aiW, M.HW[s], -Hal[s]));
+#pragma unroll
+            for (int k = 1; k < 3; k++)
+                if (k != AX) t = fma(Dup[k][s], dap[k], t);
             if (i != AX && j != AX)
-                t = i == j ? fma(sc2<2>(dal[i]), dphi[i], t)
-                           : fma(sc2<1>(dal[i]), dphi[j], fma(sc2<1>(dal[j]), dphi[i], t));
+                t = i == j ? fma(sc2<1>(dal[i]), dphi2[i], t) : fma(dal[i], dphi2[j], fma(dal[j], dphi2[i], t));
             X[s] = fma(al, Ric[s], t);
         }
         double trX = gw[0] * X[0];
@@ -978,21 +975,24 @@ __device__ __forceinline__ void rhs_core(const PointIn& P, double eta, double ou
         for (int s = 1; s < 6; s++) trX = fma(gw[s], X[s], trX);
         const double W2 = W * W;
         const double third_trX = trX * (1.0 / 3.0);
-        const double c_div = fma(-2.0 / 3.0, divbar, al * K);
+        // the term c a_ij, c = alpha K - 2/3 Dbar.beta, as c/2 of the identity in Z, then a Z and its transpose
+        const double c2 = fma(-1.0 / 3.0, divbar, 0.5 * (al * K));
+        double Y[3][3];
+#pragma unroll
+        for (int j = 0; j < 3; j++) {
+            const double z[3] = {j == 0 ? Z[0][j] + c2 : Z[0][j], j == 1 ? Z[1][j] + c2 : Z[1][j],
+                                 j == 2 ? Z[2][j] + c2 : Z[2][j]};
+#pragma unroll
+            for (int i = 0; i < 3; i++)
+                Y[i][j] = fma(a[sp(i, 2)], z[2], fma(a[sp(i, 1)], z[1], a[sp(i, 0)] * z[0]));
+        }
         double r[6];
 #pragma unroll
         for (int s = 0; s < 6; s++) {
             const int i = spi(s), j = spj(s);
-            double t = fma(a[sp(0, j)], Db[0][i], a[sp(i, 0)] * Db[0][j]);
-#pragma unroll
-            for (int k = 1; k < 3; k++) {
-                if (!dvz<FAM, AX>(k, j)) t = fma(a[sp(i, k)], Db[k][j], t);
-                if (!dvz<FAM, AX>(k, i)) t = fma(a[sp(k, j)], Db[k][i], t);
-            }
-            const double AAij = fma(a[sp(i, 2)], Aud[2][j], fma(a[sp(i, 1)], Aud[1][j], a[sp(i, 0)] * Aud[0][j]));
             const double gij = (i == j) ? 1.0 + h[s] : h[s];
             const double XTF = fma(-third_trX, gij, X[s]);
-            r[s] = fma(W2, XTF, fma(-al2, AAij, fma(c_div, a[s], t)));
+            r[s] = fma(W2, XTF, i == j ? sc2<1>(Y[i][i]) : Y[i][j] + Y[j][i]);
         }
         oms<FAM, 1>(g, vet[1], a, r);
         oms<FAM, 2>(g, vet[2], a, r);
@@ -1001,34 +1001,39 @@ __device__ __forceinline__ void rhs_core(const PointIn& P, double eta, double ou
         // Eq. W_RHS_orig_final
         out[G_CF] = (-1.0 / 3.0) * W * fma(-al, K, divbar);
         // Eq. K_RHS_orig_final
-        double lapal = gw[0] * DDal[0], gap = gw[0] * dal[0] * dphi[0];
+        // gammabar^ij Dbar_i Dbar_j alpha = gammabar^ij H_ij alpha - Delta^k e_k alpha
+        double lapal = contract6<AX>(gw, Hal), gap = gw[0] * dal[0] * dphi2[0];
+#pragma unroll
+        for (int k = 0; k < 3; k++)
+            if (k != AX) lapal = fma(-Dvec[k], dal[k], lapal);
+        // gap: 2 gammabar^ij e_i alpha e_j phi
 #pragma unroll
         for (int s = 1; s < 6; s++) {
             const int i = spi(s), j = spj(s);
-            lapal = fma(gw[s], DDal[s], lapal);
             if (i == AX || j == AX) continue;   // d_AX alpha = d_AX phi = 0
-            gap = fma(gi[s], (i == j) ? dal[i] * dphi[i] : fma(dal[i], dphi[j], dal[j] * dphi[i]), gap);
+            gap = fma(gi[s], (i == j) ? dal[i] * dphi2[i] : fma(dal[i], dphi2[j], dal[j] * dphi2[i]), gap);
         }
-        out[G_TRK] = fma(al, fma((1.0 / 3.0) * K, K, AA), -W2 * fma(2.0, gap, lapal));
+        out[G_TRK] = fma(al, fma((1.0 / 3.0) * K, K, AA), -W2 * (gap + lapal));
     }
     // Eq. Lambda_RHS_orig_final (with the alpha factors restored) + Lie terms
     double rl[3], rperp[3];
     {
         // wl_j = -2 (d_j alpha - 6 alpha d_j phi); zero along the two-point axis
-        double wl[3];
-        const double al12 = 12.0 * al;
+        double wl[3], gk[3];
+        const double al6 = 6.0 * al, al4 = sc2<2>(al);
 #pragma unroll
-        for (int k = 0; k < 3; k++) wl[k] = k == AX ? 0.0 : fma(al12, dphi[k], -sc2<1>(dal[k]));
+        for (int k = 0; k < 3; k++) {
+            wl[k] = k == AX ? 0.0 : fma(al6, dphi2[k], -sc2<1>(dal[k]));
+            gk[k] = k == AX ? gdiv[k] : fma(-al4, dK[k], gdiv[k]);   // e_k Dbar.beta - 4 alpha e_k K
+        }
 #pragma unroll
         for (int i = 0; i < 3; i++) {
-            // (2/3) Delta^i Dbar.beta + (1/3) gammabar^ik e_k Dbar.beta (the Lie-derivative part
+            // (2/3) Delta^i Dbar.beta + (1/3) gammabar^ik (e_k Dbar.beta - 4 alpha e_k K) (the Lie-derivative part
             // - lambda^j Dhat_j beta^i + beta^j (Omega_j lambda)^i is added after this block)
             double t = LapB[i];
             t = fma((2.0 / 3.0) * Dvec[i], divbar, t);
-            t = fma(1.0 / 3.0, fma(gsym(gi, i, 2), gdiv[2], fma(gsym(gi, i, 1), gdiv[1], gsym(gi, i, 0) * gdiv[0])), t);
-            // -2 Abar^ij (d_j alpha - 6 alpha d_j phi) - 4/3 alpha gammabar^ij d_j K
-            const double v = dot3<AX>(gsym(gi, i, 0), gsym(gi, i, 1), gsym(gi, i, 2), dK);
-            t = fma((-4.0 / 3.0) * al, v, t);
+            t = fma(1.0 / 3.0, fma(gsym(gi, i, 2), gk[2], fma(gsym(gi, i, 1), gk[1], gsym(gi, i, 0) * gk[0])), t);
+            // -2 Abar^ij (d_j alpha - 6 alpha d_j phi)
 #pragma unroll
             for (int k = 0; k < 3; k++)
                 if (k != AX) t = fma(Auu[sp(i, k)], wl[k], t);

@@ -44,9 +44,9 @@ __global__ void __launch_bounds__(256) k_d1(GridK G, const double* __restrict__ 
 // Bound: the FP64 pipe (2 lanes a cycle per SM: 16 to 20 cycles per warp instruction), with the difference sums on the
 // integer pipe beside it (fixed_sum.cuh).  A warp does its integer passes first and its FP64 part after
 // them; four warps per scheduler (128 registers, 3 to 5 KB of spills) keep one of them in its FP64 part nearly
-// always: 681 us per right-hand side on 256x2x512, against 693 us with three (168 registers) and 746 us with two (255
-// registers, no spills); all in FP64 arithmetic, two per scheduler: 864 us.  8th order on the same grid: 1137 -> 814
-// us; 192x96x192 spherical: 15.66 -> 11.68 ms (4th), 23.2 -> 14.5 ms (8th).
+// always: 640 us per right-hand side on 256x2x512, against 664 us with three (168 registers); two (255 registers, no
+// spills) were 10 % slower.  All in FP64 arithmetic, two per scheduler: 864 us.  8th order on the same grid: 1137 ->
+// 762 us; 192x96x192 spherical: 15.66 -> 10.45 ms (4th), 23.2 -> 12.9 ms (8th).
 constexpr int RHS_BY = 4;
 template <int FAM, int AX, int ORD>
 __global__ void __launch_bounds__(32 * RHS_BY, 4)
@@ -65,8 +65,8 @@ __global__ void __launch_bounds__(32 * RHS_BY, 4)
 }
 
 // The same for grids of few points, whose time is one warp's way through its tile: a block of SPREAD_WARPS warps
-// takes 32 consecutive interior points (i0 fastest) and divides the integer passes among its warps.  64x16x2: 93
-// -> 68 us; 72x12x24: 196 -> 168 us (with k_d1 and the launches; the all-FP64 kernel took 83 and 196 us).
+// takes 32 consecutive interior points (i0 fastest) and divides the integer passes among its warps.  64x16x2: 90
+// -> 66 us; 72x12x24: 187 -> 156 us (with k_d1 and the launches; the all-FP64 kernel took 83 and 196 us).
 // Three blocks per SM (168 registers): two are 3 % faster on the smallest grids and 35 % slower on 72x12x24, four 6
 // and 9 % slower.  It is taken up to SPREAD_TILES tiles, two rounds of three blocks on each of 152 SMs (864 tiles: 178 against 197
 // us); at 8,192 tiles it is half as fast as k_rhs, whose four warps share the FP64 pipe.
