@@ -75,7 +75,7 @@ struct Stage {
 };
 
 // Pure-outer points whose radiation condition runs inside the k_rhs launch
-// of an RK stage (extra blocks ahead of the interior tiles).
+// of an RK stage (extra blocks ahead of the interior ones).
 struct OuterArgs {
     const OuterPt* pts = nullptr;
     int npts = 0;

@@ -39,7 +39,9 @@ __global__ void __launch_bounds__(256) k_d1(GridK G, const double* __restrict__ 
 }
 
 // One RK stage (or, MODE_RHS, the right-hand side alone), one point per thread: the first oa.nblocks blocks take
-// the pure-outer points, the others tile (i0, j = i1 + N1 i2) in 32 x RHS_BY points.
+// the pure-outer points, each of the others 32 x RHS_WARPS consecutive interior points (i0 fastest), so that no lane
+// idles at the ends of rows that are no multiple of 32: 77x10x131, 8th order: 619 -> 548 us against tiles of 32 x 4
+// points, 35x2x700: 265 -> 178 us, 100x50x60: 1.24 -> 1.03 ms; rows of a multiple of 32 take the same time.
 //
 // Bound: the FP64 pipe (2 lanes a cycle per SM: 16 to 20 cycles per warp instruction), with the difference sums on the
 // integer pipe beside it (fixed_sum.cuh).  A warp does its integer passes first and its FP64 part after
@@ -47,21 +49,21 @@ __global__ void __launch_bounds__(256) k_d1(GridK G, const double* __restrict__ 
 // always: 640 us per right-hand side on 256x2x512, against 664 us with three (168 registers); two (255 registers, no
 // spills) were 10 % slower.  All in FP64 arithmetic, two per scheduler: 864 us.  8th order on the same grid: 1137 ->
 // 762 us; 192x96x192 spherical: 15.66 -> 10.45 ms (4th), 23.2 -> 12.9 ms (8th).
-constexpr int RHS_BY = 4;
+constexpr int RHS_WARPS = 4;
 template <int FAM, int AX, int ORD>
-__global__ void __launch_bounds__(32 * RHS_BY, 4)
+__global__ void __launch_bounds__(32 * RHS_WARPS, 4)
     k_rhs(GridK G, const double* __restrict__ yin, const double* __restrict__ d1x, const double* __restrict__ d1y,
           double* out, const double* yn, double* acc, Stage st, OuterArgs oa)
 {
     if ((int)blockIdx.x < oa.nblocks) {
-        const int t = blockIdx.x * (32 * RHS_BY) + threadIdx.y * 32 + threadIdx.x;
+        const int t = blockIdx.x * (32 * RHS_WARPS) + threadIdx.x;
         if (t < oa.npts)
             outer_point_stage<FAM, ORD, ssp_first_short<AX>()>(G, oa.pts[t], yin, out, yn, acc, oa.finf, oa.wspeed, st);
         return;
     }
-    const int b = blockIdx.x - oa.nblocks, nbx = (G.N0 + 31) / 32;
-    const int i = (b % nbx) * 32 + threadIdx.x, j = (b / nbx) * RHS_BY + threadIdx.y;
-    if (i < G.N0 && j < G.N1 * G.N2) rhs_point_stage<FAM, AX, ORD>(G, yin, d1x, d1y, out, yn, acc, st, i, j);
+    const int p = (blockIdx.x - oa.nblocks) * (32 * RHS_WARPS) + threadIdx.x;
+    if (p < G.N0 * G.N1 * G.N2)
+        rhs_point_stage<FAM, AX, ORD>(G, yin, d1x, d1y, out, yn, acc, st, p % G.N0, p / G.N0);
 }
 
 // The same for grids of few points, whose time is one warp's way through its tile: a block of SPREAD_WARPS warps
@@ -106,9 +108,9 @@ cudaError_t launch_k_rhs(cudaStream_t s, const GridK& G, const double* yin, doub
         k_rhs_spread<FAM, AX, ORD><<<(unsigned)(tiles + oa.nblocks), 32 * SPREAD_WARPS, 0, s>>>(G, yin, d1x, d1y, out, yn,
                                                                                               acc, st, oa);
     } else {
-        oa.nblocks = (oa.npts + 32 * RHS_BY - 1) / (32 * RHS_BY);
-        const long nb = (long)((G.N0 + 31) / 32) * (((long)G.N1 * G.N2 + RHS_BY - 1) / RHS_BY) + oa.nblocks;
-        k_rhs<FAM, AX, ORD><<<(unsigned)nb, dim3(32, RHS_BY), 0, s>>>(G, yin, d1x, d1y, out, yn, acc, st, oa);
+        oa.nblocks = (oa.npts + 32 * RHS_WARPS - 1) / (32 * RHS_WARPS);
+        const long nb = oa.nblocks + ((long)G.N0 * G.N1 * G.N2 + 32 * RHS_WARPS - 1) / (32 * RHS_WARPS);
+        k_rhs<FAM, AX, ORD><<<(unsigned)nb, 32 * RHS_WARPS, 0, s>>>(G, yin, d1x, d1y, out, yn, acc, st, oa);
     }
     return cudaGetLastError();
 }
