@@ -234,10 +234,12 @@ __host__ __device__ constexpr int d1gf(int q) { return q < 6 ? q : q == 6 ? G_CF
 // stored differences, taken beforehand on the integer pipe and read from a table (2, 3).  The second
 // differences stay in FP64: along the azimuth near the axis or a pole their rounding, at 2^-53 of f against
 // f'' dxx^2, is multiplied by 1/(dxx S)^2, so another rounding would show in the result.
-// The table lies in the thread's local memory (2) or in shared memory, [entry][lane] (3).
-enum : int { SRC_INLINE = 0, SRC_STORED = 1, SRC_TABLE = 2, SRC_SHARED = 3 };
+// The table lies in the thread's local memory (2) or in shared memory, [entry][lane] (3).  The constraints, which
+// have no stored differences, keep every first and mixed difference that they use in a table of their own (4,
+// DiagIx).
+enum : int { SRC_INLINE = 0, SRC_STORED = 1, SRC_TABLE = 2, SRC_SHARED = 3, SRC_DIAG = 4 };
 template <int S>
-__host__ __device__ constexpr bool src_table() { return S >= SRC_TABLE; }
+__host__ __device__ constexpr bool src_table() { return S == SRC_TABLE || S == SRC_SHARED; }
 template <int S>
 __host__ __device__ constexpr int src_stride() { return S == SRC_SHARED ? 32 : 1; }
 // Table index of each raw sum.  Per gridfunction with second derivatives (d1slot q): the first difference along the
@@ -254,6 +256,13 @@ struct RawIx {
     __host__ __device__ static constexpr int mix(int q, int kl) { return q * (1 + NM) + 1 + (AX < 0 ? (kl == 1 ? 0 : kl == 2 ? 1 : 2) : 0); }
     __host__ __device__ static constexpr int first(int r, int k) { return FIRST + r * NA + (AX < 0 ? k : (k == 0 ? 0 : 1)); }
     __host__ __device__ static constexpr int ox(int q) { return OX + q; }
+};
+// The constraints' table: first differences of h, a, W, K and lambda, mixed differences of h and W (slot q = 0..6).
+struct DiagIx {
+    // h, a, W, K, lambda are gridfunctions 0..16
+    __host__ __device__ static constexpr int d1(int gf, int k) { return 3 * gf + k; }
+    __host__ __device__ static constexpr int mix(int q, int kl) { return 51 + 3 * q + (kl == 1 ? 0 : kl == 2 ? 1 : 2); }
+    static constexpr int N = 51 + 21;
 };
 // r of a gridfunction with first derivatives only
 __host__ __device__ constexpr int f1slot(int gf) { return gf == G_TRK ? 3 : gf - G_LAM; }
@@ -284,6 +293,7 @@ __device__ __forceinline__ double hess(const double* f, const double* fx, const 
         constexpr int k = spi(KL), l = spj(KL);
         double m;
         if constexpr (src_table<S>()) m = rw[R::mix(q, KL) * src_stride<S>()];
+        else if constexpr (S == SRC_DIAG) m = rw[DiagIx::mix(q, KL)];
         else if constexpr (S == SRC_STORED && k == 0) m = d1r<ORD>(fx, st[l]);
         else if constexpr (S == SRC_STORED && AX < 0) m = d1r<ORD>(fy, st[l]);
         else m = mixr<ORD>(f, st[k], st[l]);
@@ -414,6 +424,7 @@ __device__ __forceinline__ double der1(const PointIn& P, int gf, int k)
 {
     if (k == AX) return 0.0;
     const int q = d1slot(gf);
+    if constexpr (S == SRC_DIAG) return P.g.D[k] * P.raw[DiagIx::d1(gf, k)];
     if (S && q >= 0 && k == 0) return P.g.D[0] * ld(P.dx + (long)q * P.T);
     if (S && AX < 0 && q >= 0 && k == 1) return P.g.D[1] * ld(P.dy + (long)q * P.T);
     if (src_table<S>())
@@ -1078,11 +1089,11 @@ __device__ __forceinline__ void rhs_core(const PointIn& P, double eta, double ou
 
 // Hamiltonian constraint, Eq. Hconstraint:
 // H = 2/3 K^2 - Abar_ij Abar^ij + W^2 (Rbar - 8 gammabar^ij d_i phi d_j phi - 8 gammabar^ij Dbar_i Dbar_j phi)
-template <int FAM, int ORD>
+template <int FAM, int ORD, int S = SRC_INLINE>
 __device__ __forceinline__ double ham_core(const PointIn& P)
 {
     MetricPart M;
-    metric_part<FAM, false, -1, SRC_INLINE, ORD>(P, M);
+    metric_part<FAM, false, -1, S, ORD>(P, M);
     const double* gi = M.gi;
     const double* gw = M.gw;
     double a[6];
@@ -1118,11 +1129,11 @@ __device__ __forceinline__ double ham_core(const PointIn& P)
 //   V_k = gammabar^jl Dhat_j a_kl - Delta^m_jk Abar^j_m - a_km Delta^m.
 // Writes the frame (rescaled) components M^i; returns |M| = sqrt(gamma_ij M^i M^j)
 // with the physical metric gamma_ij = gammabar_ij / W^2.
-template <int FAM, int ORD>
+template <int FAM, int ORD, int S = SRC_INLINE>
 __device__ __forceinline__ double mom_core(const PointIn& P, double Mv[3])
 {
     MetricPart M;
-    metric_first<FAM, -1, SRC_INLINE, ORD>(P, M);
+    metric_first<FAM, -1, S, ORD>(P, M);
     const double* y = P.y;
     const long T = P.T;
     const Geo& g = P.g;
@@ -1137,9 +1148,9 @@ __device__ __forceinline__ double mom_core(const PointIn& P, double Mv[3])
 #pragma unroll
     for (int k = 0; k < 3; k++) {
 #pragma unroll
-        for (int s = 0; s < 6; s++) Da[k][s] = g.D[k] * d1r<ORD>(F(G_ADD + s), st[k]);
-        dK[k] = g.D[k] * d1r<ORD>(F(G_TRK), st[k]);
-        dphi[k] = (-0.5 * M.iW) * (g.D[k] * d1r<ORD>(F(G_CF), st[k]));
+        for (int s = 0; s < 6; s++) Da[k][s] = der1<-1, S, ORD>(P, G_ADD + s, k);
+        dK[k] = der1<-1, S, ORD>(P, G_TRK, k);
+        dphi[k] = (-0.5 * M.iW) * der1<-1, S, ORD>(P, G_CF, k);
     }
     oms<FAM, 1>(g, a, Da[1]);   // Dhat_k a_ij
     oms<FAM, 2>(g, a, Da[2]);
@@ -1570,6 +1581,12 @@ struct FxD1 {
     }
     __device__ __forceinline__ double sum() const
     {
+        return sum([this] { return d1_fp64<ORD>(f, s); });
+    }
+    // outside: the FP64 sum, for values outside the integers' range
+    template <class Outside>
+    __device__ __forceinline__ double sum(Outside outside) const
+    {
         int k = 0;
 #pragma unroll
         for (int j = 0; j < 2 * M; j++) k = fx_max(k, fx_key(b[j]));
@@ -1595,7 +1612,7 @@ struct FxD1 {
         fx_u64 any = 0;
 #pragma unroll
         for (int j = 0; j < 2 * M; j++) any |= b[j];
-        return any << 1 ? d1_fp64<ORD>(f, s) : 0.0;
+        return any << 1 ? outside() : 0.0;
     }
 };
 
@@ -1654,6 +1671,62 @@ __device__ __forceinline__ void raw_table(const double* y, const double* d1x, co
             c = cn;
         }
     }
+}
+
+// one raw first difference (FxD1) and one mixed difference: the first difference along sb of those along sa
+template <int ORD>
+#ifdef __CUDACC__
+__noinline__
+#endif
+__device__ double fx_d1(const double* f, long s)
+{
+    FxD1<ORD> e;
+    e.f = f;
+    e.s = s;
+    e.load();
+    return e.sum();
+}
+template <int ORD>
+#ifdef __CUDACC__
+__noinline__
+#endif
+__device__ double mix_fp64(const double* f, long sa, long sb)
+{
+    return mixr<ORD>(f, sa, sb);
+}
+template <int ORD>
+__device__ __forceinline__ double fx_mix(const double* f, long sa, long sb)
+{
+    constexpr int M = FD<ORD>::M;
+    FxD1<ORD> e;
+#pragma unroll
+    for (int j = 0; j < 2 * M; j++)
+        e.b[j] = (fx_u64)__double_as_longlong(fx_d1<ORD>(f + (j < M ? j - M : j - M + 1) * sb, sa));
+    return e.sum([=] { return mix_fp64<ORD>(f, sa, sb); });
+}
+
+// the constraints' table of one point (DiagIx): first differences of gridfunctions [g0, g1) but those of [skip0,
+// skip1), and, mixed, the mixed differences
+template <int ORD>
+__device__ __forceinline__ void diag_table(const double* y, long T, const long st[3], int g0, int g1, int skip0,
+                                           int skip1, bool mixed, double* raw)
+{
+#ifdef __CUDACC__
+#pragma unroll 1
+#endif
+    for (int j = 3 * g0; j < 3 * g1; j++) {
+        const int gf = j / 3, k = j % 3;
+        if (gf >= skip0 && gf < skip1) continue;
+        raw[j] = fx_d1<ORD>(y + (long)gf * T, k == 0 ? st[0] : k == 1 ? st[1] : st[2]);
+    }
+    if (mixed)
+#ifdef __CUDACC__
+#pragma unroll 1
+#endif
+        for (int j = 0; j < 21; j++) {
+            const int m = j % 3;   // (0,1), (0,2), (1,2)
+            raw[51 + j] = fx_mix<ORD>(y + (long)d1gf(j / 3) * T, m == 2 ? st[1] : st[0], m == 0 ? st[1] : st[2]);
+        }
 }
 
 // Adds the upwinded advection and the dissipation to the 24 right-hand sides of rhs_core.

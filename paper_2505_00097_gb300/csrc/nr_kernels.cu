@@ -171,7 +171,11 @@ __global__ void k_bl(GridK G, const int* __restrict__ canon, const int* __restri
     }
 }
 
-constexpr int HAM_THREADS = 128;
+// The constraints, one point per thread: the first and mixed differences on the integer pipe into a table in local
+// memory, then the FP64 part, which bounds them (as in k_rhs).  Six blocks per SM (80 registers): both constraints
+// with their norms on 256x2x512 in 751 us, against 792 / 876 / 1063 us with four, three, two, and 904 us with the
+// differences in FP64 (no limit on the registers).
+constexpr int HAM_THREADS = 128, HAM_BLOCKS = 6;
 
 // per-block partial norms (sum of squares, max, count) of a constraint, in a fixed order
 __device__ __forceinline__ void block_partials(double s2, double mx, double cnt, double* partials)
@@ -197,7 +201,7 @@ __device__ __forceinline__ void block_partials(double s2, double mx, double cnt,
 }
 
 template <int FAM, int ORD>
-__global__ void __launch_bounds__(HAM_THREADS) k_ham(GridK G, const double* __restrict__ y, double* H, double rmin,
+__global__ void __launch_bounds__(HAM_THREADS, HAM_BLOCKS) k_ham(GridK G, const double* __restrict__ y, double* H, double rmin,
                                                       double rmax, double* partials)
 {
     const long t = (long)blockIdx.x * HAM_THREADS + threadIdx.x;
@@ -216,8 +220,11 @@ __global__ void __launch_bounds__(HAM_THREADS) k_ham(GridK G, const double* __re
         P.ox = 0;
         P.dx = nullptr;
         P.dy = nullptr;
+        double raw[DiagIx::N];
+        diag_table<ORD>(P.y, P.T, P.st, 0, G_VET, G_ADD, G_CF, true, raw);
+        P.raw = raw;
         P.g = make_geo<FAM>(G, p0, p1, p2);
-        const double h = ham_core<FAM, ORD>(P);
+        const double h = ham_core<FAM, ORD, SRC_DIAG>(P);
         if (H) H[idx] = h;
         double x[3];
         cart_of(G, p0, p1, p2, x);
@@ -234,7 +241,7 @@ __global__ void __launch_bounds__(HAM_THREADS) k_ham(GridK G, const double* __re
 // momentum constraint (Eq. Mconstraint): rescaled M^i at interior points (M: 3 gridfunctions, or
 // NULL) and per-block partial norms of |M|
 template <int FAM, int ORD>
-__global__ void __launch_bounds__(HAM_THREADS) k_mom(GridK G, const double* __restrict__ y, double* Mout, double rmin,
+__global__ void __launch_bounds__(HAM_THREADS, HAM_BLOCKS) k_mom(GridK G, const double* __restrict__ y, double* Mout, double rmin,
                                                       double rmax, double* partials)
 {
     const long t = (long)blockIdx.x * HAM_THREADS + threadIdx.x;
@@ -253,9 +260,12 @@ __global__ void __launch_bounds__(HAM_THREADS) k_mom(GridK G, const double* __re
         P.ox = 0;
         P.dx = nullptr;
         P.dy = nullptr;
+        double raw[DiagIx::N];
+        diag_table<ORD>(P.y, P.T, P.st, 0, G_LAM, 0, 0, false, raw);
+        P.raw = raw;
         P.g = make_geo<FAM>(G, p0, p1, p2);
         double Mv[3];
-        const double m = mom_core<FAM, ORD>(P, Mv);
+        const double m = mom_core<FAM, ORD, SRC_DIAG>(P, Mv);
         if (Mout) {
             Mout[idx] = Mv[0];
             Mout[G.T + idx] = Mv[1];

@@ -30,6 +30,14 @@ extern "C" void fixed_d1(int ord, const double* f, long n, double* out, double* 
     }
 }
 
+// mixed difference at the centre of an n x n block f (n = 9, axis 0 fastest), and the FP64 one
+extern "C" void fixed_mix(int ord, const double* f, double* out, double* fp64)
+{
+    const double* c = f + 4 + 9 * 4;
+    *out = ord == 8 ? fx_mix<8>(c, 1, 9) : fx_mix<4>(c, 1, 9);
+    *fp64 = ord == 8 ? mixr<8>(c, 1, 9) : mixr<4>(c, 1, 9);
+}
+
 extern "C" void fixed_sub(const double* a, const double* b, long n, double* out)
 {
     for (long i = 0; i < n; i++) out[i] = fx_sub(a[i], b[i]);

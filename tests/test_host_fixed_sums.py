@@ -84,6 +84,39 @@ def test_first_difference_outside_the_range_is_the_fp64_sum(lib, order, bad):
     assert np.array_equal(out, fp, equal_nan=True)
 
 
+@pytest.mark.parametrize("kind", ["smooth", "noise"])
+@pytest.mark.parametrize("order", [4, 8])
+def test_mixed_difference(lib, order, kind):
+    """A difference of rounded differences: each within the bound of one, and the outer one of the rounded rows."""
+    rng = np.random.default_rng(20 + order)
+    sh, weight = (5 if order == 4 else 9), sum(abs(w) for w in D1[order].values())
+    worse = 0
+    for _ in range(60):
+        f = np.ascontiguousarray(_rows(rng, kind, 1, 81).reshape(9, 9))
+        out, fp = np.empty(1), np.empty(1)
+        lib.fixed_mix(order, _p(f), _p(out), _p(fp))
+        rows = {i: sum(w * Fr(float(f[4 + i, 4 + j])) for j, w in D1[order].items()) for i in D1[order]}
+        exact = sum(w * rows[i] for i, w in D1[order].items())
+        big = Fr(float(np.abs(f).max()))
+        row = max(abs(r) for r in rows.values())
+        row_err = row / 2 ** 53 + weight * big / 2 ** (52 + sh)
+        bound = weight * row_err + (abs(exact) + weight * row_err) / 2 ** 53 + weight * (row + row_err) / 2 ** (52 + sh)
+        assert abs(Fr(float(out[0])) - exact) <= bound
+        worse += abs(Fr(float(out[0])) - exact) - abs(Fr(float(fp[0])) - exact)
+    assert worse <= 0
+
+
+@pytest.mark.parametrize("bad", [np.inf, np.nan, 1e306, 5e-324])
+@pytest.mark.parametrize("order", [4, 8])
+def test_mixed_difference_outside_the_range_is_the_fp64_one(lib, order, bad):
+    f = np.full((9, 9), bad) if abs(bad) < 1 else np.random.default_rng(2).uniform(-1, 1, (9, 9))
+    f[2, 3] = bad
+    f[6, 6] = f[6, 6] * 0.5
+    out, fp = np.empty(1), np.empty(1)
+    lib.fixed_mix(order, _p(f), _p(out), _p(fp))
+    assert np.array_equal(np.isnan(out), np.isnan(fp)) and (np.isnan(fp[0]) or out[0] == fp[0])
+
+
 def test_subtraction_is_the_ieee_difference_of_neighbours(lib):
     rng = np.random.default_rng(3)
     a = rng.uniform(-1, 1, 5000) * 2.0 ** rng.integers(-200, 200, 5000)
