@@ -1673,12 +1673,9 @@ __device__ __forceinline__ void raw_table(const double* y, const double* d1x, co
     }
 }
 
-// one raw first difference (FxD1) and one mixed difference: the first difference along sb of those along sa
+// one raw first difference (FxD1), inline and as a call
 template <int ORD>
-#ifdef __CUDACC__
-__noinline__
-#endif
-__device__ double fx_d1(const double* f, long s)
+__device__ __forceinline__ double fx_d1_inline(const double* f, long s)
 {
     FxD1<ORD> e;
     e.f = f;
@@ -1686,6 +1683,15 @@ __device__ double fx_d1(const double* f, long s)
     e.load();
     return e.sum();
 }
+template <int ORD>
+#ifdef __CUDACC__
+__noinline__
+#endif
+__device__ double fx_d1(const double* f, long s)
+{
+    return fx_d1_inline<ORD>(f, s);
+}
+// one mixed difference: the first difference along sb of those along sa; in FP64 and on the integer pipe
 template <int ORD>
 #ifdef __CUDACC__
 __noinline__
