@@ -57,12 +57,12 @@ UNIT = "point-updates/s"
 # the raw first differences counted as FP64 sums.  The kernels take those, and the advection + dissipation sums
 # (not counted here at all), in integer arithmetic beside the FP64 pipe.
 F_ALG = {"headon": 2051.3, "large3d": 2933.8, "headon8": 2493.9, "large3d8": 3719.2}
-# DRAM bytes (read + write) of the same two launches in that capture; for the large 3D grids the
-# capture's bytes per interior point at 96x48x96 (3275.7 and 5324.5, mostly register-spill lines)
+# DRAM bytes (read + write) of the k_d1 and k_rhs launches of one nr_rhs in an ncu capture; for the large 3D grids the
+# capture's bytes per interior point at 96x48x96 (6144.5 and 6816.1, mostly register-spill lines)
 # times the 28,311,552 points of the full grid
-TRAFFIC = {"headon": 24016384 + 88832 + 94202624 + 510593792,
-           "headon8": 24951296 + 119552 + 94502400 + 486498304,
-           "large3d": round(3275.7 * 28311552), "large3d8": round(5324.5 * 28311552)}
+TRAFFIC = {"headon": 24019200 + 80128 + 304581120 + 714723072,
+           "headon8": 24950016 + 105216 + 334224896 + 801484032,
+           "large3d": round(6144.5 * 28311552), "large3d8": round(6816.1 * 28311552)}
 # The same without the k_d1 pre-pass
 KERNEL_CENSUS = {"headon": 2007, "headon8": 2371, "large3d": 2844, "large3d8": 3467}
 # FLOPs over twice the FP64 instructions of the same source (k_d1 + k_rhs): the fraction of the FLOP peak
