@@ -1478,6 +1478,7 @@ __device__ __forceinline__ void adv_ko_sums(const double* y, long T, const long 
     fx_u64 ub[3], kb[2][3];
     long s[3];
     int key = 0;
+    fx_u64 any = 0;
 #pragma unroll
     for (int d = 0; d < 3; d++) {
         const double v = ld(y + (long)(G_VET + d) * T);
@@ -1490,7 +1491,9 @@ __device__ __forceinline__ void adv_ko_sums(const double* y, long T, const long 
         kb[0][d] = (fx_u64)__double_as_longlong(kc * sigma_metric * D[d]);
         kb[1][d] = (fx_u64)__double_as_longlong(kc * sigma_gauge * D[d]);
         key = fx_max(key, fx_max(fx_key(ub[d]), fx_max(fx_key(kb[0][d]), fx_key(kb[1][d]))));
+        any |= ub[d] | kb[0][d] | kb[1][d];
     }
+    const bool none = !(any << 1);   // no shift and no dissipation
     const int Ec = key >> 20;
     FxSplit cu[3], ck[2][3];
 #pragma unroll
@@ -1545,8 +1548,8 @@ __device__ __forceinline__ void adv_ko_sums(const double* y, long T, const long 
                 fx_mac(dot, kap, fx_split(K));
             }
             r = fx_out2(dot.hh, dot.cross, E + Ec - 2 * 1075 - F::SH - F::SC + F::Q + 32);
-        } else if (okc && in.zero()) {
-            r = 0.0;   // all values zero: the sum is zero for any finite weights
+        } else if ((okc && in.zero()) || (none && E < 2047)) {
+            r = 0.0;   // all values zero and finite weights, or the reverse
         } else {
             r = advko_fp64<AX, ORD>(f, st, ox, u, fwd, D, g < G_VET ? sigma_metric : sigma_gauge);
         }

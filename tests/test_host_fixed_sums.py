@@ -199,3 +199,16 @@ def test_advection_outside_the_range_is_the_fp64_sum(lib, order, where, bad):
     out, fp = np.empty(1), np.empty(1)
     lib.fixed_advko(-1, order, _p(f), _p(vet), _p(D), ctypes.c_double(0.3), _p(out), _p(fp))
     assert np.array_equal(out, fp, equal_nan=True)
+
+
+@pytest.mark.parametrize("value", [1.0, np.inf, np.nan])
+@pytest.mark.parametrize("ax", [-1, 1])
+@pytest.mark.parametrize("order", [4, 8])
+def test_no_shift_and_no_dissipation(lib, order, ax, value):
+    """Zero weights: zero, or the NaN of the FP64 sum where a value is not finite."""
+    f = np.ascontiguousarray(np.random.default_rng(6).uniform(-1, 1, (11, 11, 11)))
+    f[5, 5, 6] = value
+    out, fp = np.empty(1), np.empty(1)
+    lib.fixed_advko(ax, order, _p(f), _p(np.zeros(3)), _p(np.array([3.0, 1.0, 2.0])), ctypes.c_double(0.0), _p(out), _p(fp))
+    assert np.array_equal(out, fp, equal_nan=True)
+    assert (out[0] == 0.0) == bool(np.isfinite(value))
