@@ -1569,8 +1569,9 @@ __device__ double d1_fp64(const double* f, long s)
 }
 
 // The raw first difference of f along stride s, exact up to the alignment of the values to the largest of them and
-// rounded once.  4th order: a sum within 64 bits (weights up to 18 in all, 5 guard bits); 8th order: in two
-// words (weights up to 1750, 9 guard bits).  load() reads the values, sum() adds them up.
+// rounded once.  4th order: a sum within 64 bits (weights up to 18 in all, 5 guard bits: 18 x 2^58 < 2^63); 8th order: in
+// two words (weights up to 1750, 9 guard bits: values below 2^62, their differences below 2^63).  load() reads the
+// values, sum() adds them up.
 template <int ORD>
 struct FxD1 {
     static constexpr int M = FD<ORD>::M, SH = ORD == 4 ? 5 : 9;
@@ -1601,15 +1602,18 @@ struct FxD1 {
             if constexpr (ORD == 4) {
                 return fx_out(8 * d[0] - d[1], E - 1075 - SH);
             } else {
+                // |d| reaches 2^63 - 2^10, beyond fx_split: the low words are taken unsigned, d = h 2^32 + l with
+                // h = floor(d / 2^32), which holds for every d
                 constexpr int w[4] = {672, -168, 32, -3};
-                fx_i64 h = 0, l = 0;
+                fx_i64 h = 0;
+                fx_u64 l = 0;   // modulo 2^64: the sum lies within +-704 x 2^32
 #pragma unroll
                 for (int o = 0; o < M; o++) {
-                    const FxSplit m = fx_split(d[o]);
-                    h += (fx_i64)m.h * w[o];
-                    l += (fx_i64)m.l * w[o];
+                    h += (fx_i64)(int)(d[o] >> 32) * w[o];
+                    if (w[o] > 0) l += (fx_u64)(unsigned)d[o] * (unsigned)w[o];
+                    else l -= (fx_u64)(unsigned)d[o] * (unsigned)-w[o];
                 }
-                return fx_out2(h, l, E - 1075 - SH);
+                return fx_out2(h, (fx_i64)l, E - 1075 - SH);
             }
         }
         fx_u64 any = 0;

@@ -46,7 +46,8 @@ __device__ __forceinline__ fx_i64 fx_in(fx_u64 b, int E)
     return (fx_i64)((a ^ (fx_u64)s) - (fx_u64)s);
 }
 
-// m = h 2^32 + l with l signed: products of the parts are signed 32 x 32 -> 64 multiplies
+// m = h 2^32 + l with l signed: products of the parts are signed 32 x 32 -> 64 multiplies.  m < 2^63 - 2^31, above which
+// the carry of a negative l takes h out of 32 bits.
 struct FxSplit {
     int h, l;
 };
