@@ -56,7 +56,7 @@ UNIT = "point-updates/s"
 # as the point code's source has them (add + mul + div + 2 fma, a host census that a test recomputes), with
 # the raw first differences counted as FP64 sums.  The kernels take those, and the advection + dissipation sums
 # (not counted here at all), in integer arithmetic beside the FP64 pipe.
-F_ALG = {"headon": 2051.3, "large3d": 2933.8, "headon8": 2493.9, "large3d8": 3719.2}
+F_ALG = {"headon": 2071.3, "large3d": 2963.8, "headon8": 2513.9, "large3d8": 3749.2}
 # DRAM bytes (read + write) of the k_d1 and k_rhs launches of one nr_rhs in an ncu capture; for the large 3D grids the
 # capture's bytes per interior point at 96x48x96 (6144.5 and 6816.1, mostly register-spill lines)
 # times the 28,311,552 points of the full grid
@@ -64,24 +64,23 @@ TRAFFIC = {"headon": 24019200 + 80128 + 304581120 + 714723072,
            "headon8": 24950016 + 105216 + 334224896 + 801484032,
            "large3d": round(6144.5 * 28311552), "large3d8": round(6816.1 * 28311552)}
 # The same without the k_d1 pre-pass
-KERNEL_CENSUS = {"headon": 2007, "headon8": 2371, "large3d": 2844, "large3d8": 3467}
+KERNEL_CENSUS = {"headon": 2027, "headon8": 2391, "large3d": 2874, "large3d8": 3497}
 # FLOPs over twice the FP64 instructions of the same source (k_d1 + k_rhs): the fraction of the FLOP peak
 # that a fully busy FP64 pipe reaches with this mix (a DADD or DMUL takes an FMA's issue slot for 1 FLOP)
-MIX_CEILING = {"headon": 0.7810, "headon8": 0.7653, "large3d": 0.7906, "large3d8": 0.7696}
+MIX_CEILING = {"headon": 0.7827, "headon8": 0.7667, "large3d": 0.7923, "large3d8": 0.7710}
 # FP64 operations (add + mul + div) per interior point of one RHS evaluation as the oracle's counting
 # build counts them: the plain coordinate-basis evaluation of the same discretisation with generic index
 # loops and the reference metric evaluated at every point -- the work of the method evaluated plainly.
 # Achieved against it (frac_method) can exceed 1: the kernels compute the same discrete right-hand side
 # with about a tenth of those operations
 F_METHOD = {"headon": 28967, "headon8": 49631, "large3d": 28970, "large3d8": 49634}
-# The same for the diagnostics (Hamiltonian and momentum constraints, psi4), per interior
-# point of one call, from one ncu capture of those kernels on the head-on state, by workload
-# (head-on: k_ham 363 / 218 / 593 DADD / DMUL / DFMA, k_mom 111 / 142 / 262, k_psi4 460 / 434 /
-# 1016; the reductions and ghost copies add < 0.1); absent: not captured
-DIAG_FLOPS = {"headon": {"hamiltonian": 1767.0, "momentum": 777.0, "psi4": 2926.0}}
-# the source census of the constraints' point code those counts were taken with (FMA = 2, one division,
-# the square root of |M| not counted: its expansion is most of the 34 FLOP the momentum count adds)
-DIAG_CENSUS = {"headon": {"hamiltonian": 1773, "momentum": 743}}
+# The same for the diagnostics, per interior point of one call, by workload: the constraints' FP64 operations as the
+# point code's source has them (a host census that a test recomputes: FMA = 2, one division, the square root of |M| not
+# counted; their first and mixed differences counted as FP64 sums, which the kernels take on the integer pipe), psi4's
+# from an ncu capture of k_psi4 (460 / 434 / 1016 DADD / DMUL / DFMA); absent: not counted
+DIAG_FLOPS = {"headon": {"hamiltonian": 1767.0, "momentum": 737.0, "psi4": 2926.0}}
+# the census alone
+DIAG_CENSUS = {"headon": {"hamiltonian": 1767, "momentum": 737}}
 # psi4 modes on the workload's extraction sphere: l <= 8, Gauss-Legendre x uniform nodes
 PSI4_LMAX, PSI4_NTHETA, PSI4_NPHI = 8, 24, 48
 # FP64 pipe of one SM: 2 DFMA per clock (ncu peak_sustained of

@@ -452,7 +452,6 @@ struct MetricPart {
     double Dl2[3][6];    // 2 Delta_kij (first index lowered)
     double Dup[3][6];    // Delta^k_ij
     double Dvec[3];      // Delta^k
-    double Dtr[3];       // Delta^k_km
     double Ric[6];       // Rbar_ij
     double W, iW, dphi[3];
     double HW[6];        // H_ij W (right-hand side)
@@ -460,8 +459,8 @@ struct MetricPart {
 };
 
 // The conformal metric and its inverse, first frame derivatives of h, and
-// Delta (lowered, raised, its trace Delta^k and Delta^k_km): shared by the
-// right-hand side and both constraints.
+// Delta (lowered, raised, its trace Delta^k): shared by the right-hand side and
+// both constraints.
 template <int FAM, int AX, int S, int ORD>
 __device__ __forceinline__ void metric_first(const PointIn& P, MetricPart& M)
 {
@@ -542,9 +541,25 @@ __device__ __forceinline__ void metric_first(const PointIn& P, MetricPart& M)
         for (int s = 1; s < 6; s++) t = fma(gw[s], Dup[k][s], t);
         Dvec[k] = t;
     }
-    // Delta^k_km (= 1/2 gammabar^ab e_m h_ab: zero along the two-point axis)
+}
+
+// Delta^k_km = 1/2 gammabar^ab e_m h_ab (zero along the two-point axis).  Not the trace of Delta^k_ij, which would take
+// two additions: its terms hold the rotation of h, which cancels in the sum only, and the error of d_t W then
+// grows with the stretch of the metric (3 to 19 times at an eigenvalue ratio of 101).
+template <int AX>
+__device__ __forceinline__ void delta_trace(const MetricPart& M, double Dtr[3])
+{
 #pragma unroll
-    for (int m = 0; m < 3; m++) M.Dtr[m] = m == AX ? 0.0 : Dup[0][sp(0, m)] + Dup[1][sp(1, m)] + Dup[2][sp(2, m)];
+    for (int m = 0; m < 3; m++) {
+        if (m == AX) {
+            Dtr[m] = 0.0;
+            continue;
+        }
+        double t = M.gw[0] * M.dh[m][0];
+#pragma unroll
+        for (int s = 1; s < 6; s++) t = fma(M.gw[s], M.dh[m][s], t);
+        Dtr[m] = sc2<-1>(t);
+    }
 }
 
 template <int FAM, bool NEED_GH, int AX, int S, int ORD>
@@ -735,7 +750,8 @@ __device__ __forceinline__ void rhs_core(const PointIn& P, double eta, double ou
     const double (*dh)[6] = M.dh;
     const double (*Dup)[6] = M.Dup;
     const double* Dvec = M.Dvec;
-    const double* Dtr = M.Dtr;
+    double Dtr[3];   // Delta^k_km
+    delta_trace<AX>(M, Dtr);
     const double* GH = M.GH;
     const double* Ric = M.Ric;
     const double W = M.W;
