@@ -1758,6 +1758,18 @@ __device__ __forceinline__ void diag_table(const double* y, long T, const long s
         }
 }
 
+// the tables that the Hamiltonian and the momentum constraint read
+template <int ORD>
+__device__ __forceinline__ void ham_table(const PointIn& P, double raw[DiagIx::N])
+{
+    diag_table<ORD>(P.y, P.T, P.st, 0, G_VET, G_ADD, G_CF, true, raw);
+}
+template <int ORD>
+__device__ __forceinline__ void mom_table(const PointIn& P, double raw[DiagIx::N])
+{
+    diag_table<ORD>(P.y, P.T, P.st, 0, G_LAM, 0, 0, false, raw);
+}
+
 // Adds the upwinded advection and the dissipation to the 24 right-hand sides of rhs_core.
 template <int AX, int ORD>
 __device__ __forceinline__ void add_adv_ko(const double* y, long T, const long st[3], long ox, const double D[3],

@@ -221,7 +221,7 @@ __global__ void __launch_bounds__(HAM_THREADS, HAM_BLOCKS) k_ham(GridK G, const 
         P.dx = nullptr;
         P.dy = nullptr;
         double raw[DiagIx::N];
-        diag_table<ORD>(P.y, P.T, P.st, 0, G_VET, G_ADD, G_CF, true, raw);
+        ham_table<ORD>(P, raw);
         P.raw = raw;
         P.g = make_geo<FAM>(G, p0, p1, p2);
         const double h = ham_core<FAM, ORD, SRC_DIAG>(P);
@@ -261,7 +261,7 @@ __global__ void __launch_bounds__(HAM_THREADS, HAM_BLOCKS) k_mom(GridK G, const 
         P.dx = nullptr;
         P.dy = nullptr;
         double raw[DiagIx::N];
-        diag_table<ORD>(P.y, P.T, P.st, 0, G_LAM, 0, 0, false, raw);
+        mom_table<ORD>(P, raw);
         P.raw = raw;
         P.g = make_geo<FAM>(G, p0, p1, p2);
         double Mv[3];
