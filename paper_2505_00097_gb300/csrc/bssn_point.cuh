@@ -76,20 +76,6 @@ __device__ __forceinline__ double mixraw(const double* f, long sa, long sb)
     double p1 = d1raw(f + sb, sa), p2 = d1raw(f + 2 * sb, sa);
     return fma(8.0, p1 - m1, m2 - p2);
 }
-// upwind-biased: -3 g[-1] - 10 g[0] + 18 g[1] - 6 g[2] + g[3], g[o] = f[o*s]
-// (s = -stride gives the mirrored stencil up to an overall sign)
-__device__ __forceinline__ double upraw(const double* f, long s)
-{
-    double t1 = fma(-3.0, ld(f - s), ld(f + 3 * s));
-    double t2 = fma(3.0, ld(f + s), -ld(f + 2 * s));
-    return fma(-10.0, ld(f), fma(6.0, t2, t1));
-}
-// sixth difference without its centre term: (f-3+f3) - 6 (f-2+f2) + 15 (f-1+f1)
-__device__ __forceinline__ double koraw(const double* f, long s)
-{
-    return fma(15.0, ld(f - s) + ld(f + s), fma(-6.0, ld(f - 2 * s) + ld(f + 2 * s), ld(f - 3 * s) + ld(f + 3 * s)));
-}
-
 // ---- 8th-order stencils (the production scheme of Sec. 4.1, N_G = 5), integer
 // weights: first derivative over 840 h, second over 5040 h^2 (the scale factors
 // are in Geo); a mixed derivative is the first-derivative stencil applied to the
