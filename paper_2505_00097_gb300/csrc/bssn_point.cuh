@@ -1720,18 +1720,17 @@ __device__ __forceinline__ double fx_mix(const double* f, long sa, long sb)
     return e.sum([=] { return mix_fp64<ORD>(f, sa, sb); });
 }
 
-// the constraints' table of one point (DiagIx): first differences of gridfunctions [g0, g1) but those of [skip0,
-// skip1), and, mixed, the mixed differences
-template <int ORD>
-__device__ __forceinline__ void diag_table(const double* y, long T, const long st[3], int g0, int g1, int skip0,
-                                           int skip1, bool mixed, double* raw)
+// the constraints' table of one point (DiagIx): first differences of the gridfunctions with their bit set in GFS and,
+// mixed, the mixed differences
+template <int ORD, unsigned GFS>
+__device__ __forceinline__ void diag_table(const double* y, long T, const long st[3], bool mixed, double* raw)
 {
 #ifdef __CUDACC__
 #pragma unroll 1
 #endif
-    for (int j = 3 * g0; j < 3 * g1; j++) {
+    for (int j = 0; j < 3 * G_VET; j++) {
         const int gf = j / 3, k = j % 3;
-        if (gf >= skip0 && gf < skip1) continue;
+        if (!(GFS >> gf & 1)) continue;
         raw[j] = fx_d1<ORD>(y + (long)gf * T, k == 0 ? st[0] : k == 1 ? st[1] : st[2]);
     }
     if (mixed)
@@ -1743,17 +1742,18 @@ __device__ __forceinline__ void diag_table(const double* y, long T, const long s
             raw[51 + j] = fx_mix<ORD>(y + (long)d1gf(j / 3) * T, m == 2 ? st[1] : st[0], m == 0 ? st[1] : st[2]);
         }
 }
-
-// the tables that the Hamiltonian and the momentum constraint read
+// the tables that the Hamiltonian (h, W, lambda; K has no derivative in it) and the momentum constraint (h, a, W, K) read
 template <int ORD>
 __device__ __forceinline__ void ham_table(const PointIn& P, double raw[DiagIx::N])
 {
-    diag_table<ORD>(P.y, P.T, P.st, 0, G_VET, G_ADD, G_CF, true, raw);
+    constexpr unsigned h = 0x3Fu << G_HDD, lam = 7u << G_LAM;
+    diag_table<ORD, h | 1u << G_CF | lam>(P.y, P.T, P.st, true, raw);
 }
 template <int ORD>
 __device__ __forceinline__ void mom_table(const PointIn& P, double raw[DiagIx::N])
 {
-    diag_table<ORD>(P.y, P.T, P.st, 0, G_LAM, 0, 0, false, raw);
+    constexpr unsigned h = 0x3Fu << G_HDD, a = 0x3Fu << G_ADD;
+    diag_table<ORD, h | a | 1u << G_CF | 1u << G_TRK>(P.y, P.T, P.st, false, raw);
 }
 
 // Adds the upwinded advection and the dissipation to the 24 right-hand sides of rhs_core.
