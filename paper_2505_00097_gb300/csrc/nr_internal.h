@@ -84,11 +84,19 @@ struct OuterArgs {
     const double* wspeed = nullptr;
 };
 
+// What runs at the same time as a launch of k_rhs, itself included: tiles of 32 interior points, summed over the grids or
+// partitions whose launches are parallel branches, on a device of n_sm SMs.
+struct RhsLoad {
+    int n_sm = 0;
+    long tiles = 0;
+    void add(const GridK& G) { tiles += ((long)G.N0 * G.N1 * G.N2 + 31) / 32; }
+};
+
 // kernel launchers (nr_kernels.cu)
 // k_d1 on yin into d1x / d1y (N_D1 sets of T doubles each; d1y used on general
 // grids only), then k_rhs
 cudaError_t launch_rhs(const GridK& G, const double* yin, double* d1x, double* d1y, double* out, const double* yn,
-                       double* acc, Stage st, cudaStream_t s, OuterArgs oa = OuterArgs());
+                       double* acc, Stage st, cudaStream_t s, const RhsLoad& load, OuterArgs oa = OuterArgs());
 cudaError_t launch_outer(const GridK& G, const OuterPt* pts, int npts, const double* yin, double* out,
                          const double* yn, double* acc, const double* finf, const double* wspeed, Stage st,
                          cudaStream_t s);
@@ -160,6 +168,7 @@ struct nr_grid {
     cudaStream_t stream = nullptr;   // user stream (may be the legacy stream)
     cudaStream_t cap = nullptr;      // internal stream used for graph capture
     int device = 0;
+    nrk::RhsLoad load;
     // device buffers
     double *y = nullptr, *ya = nullptr, *yb = nullptr, *acc = nullptr;
     double *ax0 = nullptr, *ax1 = nullptr, *ax2 = nullptr;

@@ -70,9 +70,10 @@ __global__ void __launch_bounds__(32 * RHS_WARPS, 4)
 // takes 32 consecutive interior points (i0 fastest) and divides the integer passes among its warps.  64x16x2: 90
 // -> 66 us; 72x12x24: 187 -> 156 us (with k_d1 and the launches; the all-FP64 kernel took 83 and 196 us).
 // Three blocks per SM (168 registers): two are 3 % faster on the smallest grids and 35 % slower on 72x12x24, four 6
-// and 9 % slower.  It is taken up to SPREAD_TILES tiles, two rounds of three blocks on each of 152 SMs (864 tiles: 178 against 197
-// us); at 8,192 tiles it is half as fast as k_rhs, whose four warps share the FP64 pipe.
-constexpr long SPREAD_TILES = 2 * 3 * 152;
+// and 9 % slower.  It is taken up to two rounds of three blocks per SM (864 tiles: 178 against 197 us), counting the
+// tiles of every launch that runs at once; at 8,192 tiles it is half as fast as k_rhs, whose four warps share the
+// FP64 pipe (256x2x512 in 16 partitions of 512 tiles: an RK4 step of 4.71 against 3.57 ms).
+constexpr long SPREAD_TILES_PER_SM = 2 * 3;
 template <int FAM, int AX, int ORD>
 __global__ void __launch_bounds__(32 * SPREAD_WARPS, 3)
     k_rhs_spread(GridK G, const double* __restrict__ yin, const double* __restrict__ d1x,
@@ -100,10 +101,10 @@ __global__ void __launch_bounds__(32 * SPREAD_WARPS, 3)
 
 template <int FAM, int AX, int ORD>
 cudaError_t launch_k_rhs(cudaStream_t s, const GridK& G, const double* yin, double* d1x, double* d1y, double* out,
-                         const double* yn, double* acc, const Stage& st, OuterArgs oa)
+                         const double* yn, double* acc, const Stage& st, const RhsLoad& load, OuterArgs oa)
 {
     const long tiles = ((long)G.N0 * G.N1 * G.N2 + 31) / 32;
-    if (tiles <= SPREAD_TILES) {
+    if (load.tiles <= SPREAD_TILES_PER_SM * load.n_sm) {
         oa.nblocks = (oa.npts + 32 * SPREAD_WARPS - 1) / (32 * SPREAD_WARPS);
         k_rhs_spread<FAM, AX, ORD><<<(unsigned)(tiles + oa.nblocks), 32 * SPREAD_WARPS, 0, s>>>(G, yin, d1x, d1y, out, yn,
                                                                                               acc, st, oa);
@@ -370,7 +371,7 @@ cudaError_t launch_fp64_probe(int blocks, int iters, double* sink, cudaStream_t 
 
 template <int ORD>
 cudaError_t launch_rhs_ord(const GridK& G, const double* yin, double* d1x, double* d1y, double* out,
-                           const double* yn, double* acc, Stage st, cudaStream_t s, OuterArgs oa)
+                           const double* yn, double* acc, Stage st, cudaStream_t s, const RhsLoad& load, OuterArgs oa)
 {
     // the stored first differences of yin
     {
@@ -382,18 +383,18 @@ cudaError_t launch_rhs_ord(const GridK& G, const double* yin, double* d1x, doubl
         if (e != cudaSuccess) return e;
     }
     if (G.fam == FAM_SPH) {
-        if (G.ax == 2) return launch_k_rhs<FAM_SPH, 2, ORD>(s, G, yin, d1x, d1y, out, yn, acc, st, oa);
-        return launch_k_rhs<FAM_SPH, -1, ORD>(s, G, yin, d1x, d1y, out, yn, acc, st, oa);
+        if (G.ax == 2) return launch_k_rhs<FAM_SPH, 2, ORD>(s, G, yin, d1x, d1y, out, yn, acc, st, load, oa);
+        return launch_k_rhs<FAM_SPH, -1, ORD>(s, G, yin, d1x, d1y, out, yn, acc, st, load, oa);
     }
-    if (G.ax == 1) return launch_k_rhs<FAM_CYL, 1, ORD>(s, G, yin, d1x, d1y, out, yn, acc, st, oa);
-    return launch_k_rhs<FAM_CYL, -1, ORD>(s, G, yin, d1x, d1y, out, yn, acc, st, oa);
+    if (G.ax == 1) return launch_k_rhs<FAM_CYL, 1, ORD>(s, G, yin, d1x, d1y, out, yn, acc, st, load, oa);
+    return launch_k_rhs<FAM_CYL, -1, ORD>(s, G, yin, d1x, d1y, out, yn, acc, st, load, oa);
 }
 
 cudaError_t launch_rhs(const GridK& G, const double* yin, double* d1x, double* d1y, double* out, const double* yn,
-                       double* acc, Stage st, cudaStream_t s, OuterArgs oa)
+                       double* acc, Stage st, cudaStream_t s, const RhsLoad& load, OuterArgs oa)
 {
-    return G.ord == 8 ? launch_rhs_ord<8>(G, yin, d1x, d1y, out, yn, acc, st, s, oa)
-                      : launch_rhs_ord<4>(G, yin, d1x, d1y, out, yn, acc, st, s, oa);
+    return G.ord == 8 ? launch_rhs_ord<8>(G, yin, d1x, d1y, out, yn, acc, st, s, load, oa)
+                      : launch_rhs_ord<4>(G, yin, d1x, d1y, out, yn, acc, st, s, load, oa);
 }
 
 cudaError_t launch_outer(const GridK& G, const OuterPt* pts, int npts, const double* yin, double* out,

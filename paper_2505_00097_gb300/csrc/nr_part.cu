@@ -281,6 +281,7 @@ struct nr_part {
     nr_params P;
     HostGeom G;
     GridK K;   // the whole grid's kernel description (no device arrays)
+    RhsLoad load;   // all partitions together
     double dt_cfl = 0.0;
     int parts[3] = {1, 1, 1};
     int device = 0;
@@ -404,7 +405,7 @@ int enqueue_stage(nr_part* s, cudaStream_t st, int in, int out, const Stage& sg,
         oa.finf = s->finf;
         oa.wspeed = s->wspeed;
         PCUDA(launch_rhs(d.K, buf_of(d, in), d.d1x, d.d1y, buf_of(d, out), yn_is_y ? d.y : nullptr,
-                         use_acc ? d.acc : nullptr, sg, ps, oa));
+                         use_acc ? d.acc : nullptr, sg, ps, s->load, oa));
         PCUDA(launch_inner(d.K, d.inner, d.n_inner, buf_of(d, out), ps));
         if (forked) {
             PCUDA(cudaEventRecord(s->pevent[q], ps));
@@ -583,7 +584,10 @@ static int nr_part_create_body(int coords, const int Nxx[3], const nr_params* pa
                     return rc;
                 }
             }
-        cudaError_t e = cudaStreamCreateWithFlags(&s->cap, cudaStreamNonBlocking);
+        // the partitions' kernels are parallel branches of the captured step
+        for (PartDev& d : s->p) s->load.add(d.K);
+        cudaError_t e = cudaDeviceGetAttribute(&s->load.n_sm, cudaDevAttrMultiProcessorCount, s->device);
+        if (e == cudaSuccess) e = cudaStreamCreateWithFlags(&s->cap, cudaStreamNonBlocking);
         if (e == cudaSuccess) e = cudaEventCreateWithFlags(&s->fork, cudaEventDisableTiming);
         s->pstream.assign(s->p.size(), nullptr);
         s->pevent.assign(s->p.size(), nullptr);
