@@ -677,7 +677,7 @@ int nrk::grid_from_setup(HostSetup& H, const nr_params& P, nr_grid** out)
         if (e == cudaSuccess) e = cudaMemset(g->acc, 0, sizeof(double) * set);
         if (e == cudaSuccess) e = cudaStreamCreateWithFlags(&g->cap, cudaStreamNonBlocking);
         if (e == cudaSuccess) e = cudaDeviceGetAttribute(&g->load.n_sm, cudaDevAttrMultiProcessorCount, g->device);
-        g->load.add(K);
+        g->load.add(K, g->n_outer);
         if (e != cudaSuccess) {
             free_grid(g);
             return fail(NR_ECUDA, "grid upload: %s", cudaGetErrorString(e));
@@ -763,7 +763,9 @@ int nr_rhs(nr_grid* g, const double* y_dev, double* rhs_dev)
     if (!g || !y_dev || !rhs_dev || y_dev == rhs_dev) return fail(NR_EINVAL, "bad nr_rhs arguments");
     DeviceGuard dg(g->device);
     Stage st{MODE_RHS, 0, 0.0, 0.0, 0.0};
-    CUDA_OR_FAIL(launch_rhs(g->K, y_dev, g->d1x, g->d1y, rhs_dev, nullptr, nullptr, st, g->stream, g->load));
+    RhsLoad load = g->load;
+    load.outer = 0;
+    CUDA_OR_FAIL(launch_rhs(g->K, y_dev, g->d1x, g->d1y, rhs_dev, nullptr, nullptr, st, g->stream, load));
     return NR_OK;
 }
 

@@ -75,7 +75,7 @@ struct Stage {
 };
 
 // Pure-outer points whose radiation condition runs inside the k_rhs launch
-// of an RK stage (extra blocks ahead of the interior ones).
+// of an RK stage (extra blocks ahead of the interior ones or behind them).
 struct OuterArgs {
     const OuterPt* pts = nullptr;
     int npts = 0;
@@ -84,13 +84,44 @@ struct OuterArgs {
     const double* wspeed = nullptr;
 };
 
-// What runs at the same time as a launch of k_rhs, itself included: tiles of 32 interior points, summed over the grids or
-// partitions whose launches are parallel branches, on a device of n_sm SMs.
+// What runs at the same time as a launch of k_rhs, itself included: tiles of 32 interior points and blocks of 128
+// pure-outer points, summed over the grids or partitions whose launches are parallel branches, on a device of n_sm
+// SMs.
 struct RhsLoad {
     int n_sm = 0;
-    long tiles = 0;
-    void add(const GridK& G) { tiles += ((long)G.N0 * G.N1 * G.N2 + 31) / 32; }
+    long tiles = 0, outer = 0;
+    void add(const GridK& G, int n_outer)
+    {
+        tiles += ((long)G.N0 * G.N1 * G.N2 + 31) / 32;
+        outer += (n_outer + 127) / 128;
+    }
 };
+
+// The launch shape of the right-hand side (nr_rhs_kernels.cuh): tiles of 32 points spread over four warps, three or four
+// blocks per SM, or one point per thread, two or four blocks of 128 per SM.  A launch of few blocks takes
+// about as long as its fullest SM, so the lines lie where a round is full, counted in the device's SMs.  us per RK step on
+// a GB300 (152 SMs) beside the other shapes, and beside the all-FP64 kernel of one point per thread; cyl2 = 64x2xN,
+// cyl = 64x8xN cylindrical, sph2 = 64xNx2, sph = 64x16xN spherical:
+//   one round of three spread blocks: cyl2, 304 tiles: 264, four 274, points 326 (two) and 352 (four), all-FP64 318
+//   one round of four: cyl2, 520 tiles: 311, three 462, points 327 and 352, all-FP64 319; sph, 576: 423, 653, 464, 531, 443.
+//     Not with two-point azimuth and 8th order, where the integer part outweighs the FP64 part: cyl2, 520: points 295,
+//     four 354, all-FP64 301; sph2, 520: 319, 342, 326
+//   two rounds of three: cyl2, 760: 476, points 504 and 524, all-FP64 543; sph, 640: 656, 700, 754, 750; a third round
+//     loses: cyl2, 912: 621 against 505
+//   two blocks of 128 per SM: cyl2, 1064: 509, four 546, all-FP64 553; sph, 1216: 852, 1043, 861.  The outer blocks of
+//     the 8th order are as long as tiles and count: cyl2, 1184, 8th: 719, four 657
+//   outer blocks alone would put a fourth block on an SM, 4th order: cyl2, 1824: 811, four 925, all-FP64 902
+enum RhsShape { RHS_SPREAD3, RHS_SPREAD4, RHS_POINTS2, RHS_POINTS4 };
+inline RhsShape rhs_shape(int ord, bool two_point, const RhsLoad& l)
+{
+    const long sm = l.n_sm, all = l.tiles + l.outer, blocks = (l.tiles + 3) / 4;
+    if (all <= 3 * sm) return RHS_SPREAD3;
+    if (all <= 4 * sm && !(two_point && ord == 8)) return RHS_SPREAD4;
+    if (l.tiles > 4 * sm && all <= 6 * sm) return RHS_SPREAD3;
+    if (blocks + (ord == 8 ? l.outer : 0) <= 2 * sm) return RHS_POINTS2;
+    if (ord == 4 && blocks <= 3 * sm && blocks + l.outer > 3 * sm) return RHS_POINTS2;
+    return RHS_POINTS4;
+}
 
 // kernel launchers (nr_kernels.cu)
 // k_d1 on yin into d1x / d1y (N_D1 sets of T doubles each; d1y used on general

@@ -2,11 +2,12 @@
 //
 //   k_d1      raw first differences along axes 0 (and 1) of the gridfunctions
 //             with second derivatives, read by k_rhs for its mixed derivatives
-//   k_rhs     interior right-hand side (Sec. 2.1 equations, upwinded advection,
-//             Kreiss-Oliger dissipation) with the RK4 stage update and the
-//             det(gammabar) enforcement fused into its epilogue; in an RK
-//             stage its first blocks also run the radiation condition at the
-//             pure-outer ghosts (Sec. 3) with the same epilogue
+//   k_rhs     (nr_rhs_kernels.cuh, launched from here) interior right-hand side
+//             (Sec. 2.1 equations, upwinded advection, Kreiss-Oliger dissipation)
+//             with the RK4 stage update and the det(gammabar) enforcement fused
+//             into its epilogue; in an RK stage some of its blocks run the
+//             radiation condition at the pure-outer ghosts (Sec. 3) with the same
+//             epilogue
 //   k_outer   the radiation condition alone (nr_apply_bcs)
 //   k_inner   parity copies at inner ghosts (Sec. 3), one warp-coalesced gather
 //             per gridfunction
@@ -23,6 +24,7 @@
 #include "bssn_point.cuh"
 #include "nr_geo.cuh"
 #include "nr_internal.h"
+#include "nr_rhs_kernels.cuh"
 #include "nr_stage.cuh"
 
 namespace nrk {
@@ -36,84 +38,6 @@ template <int AX, int ORD>
 __global__ void __launch_bounds__(256) k_d1(GridK G, const double* __restrict__ y, double* d1x, double* d1y)
 {
     d1_point<AX, ORD>(G, y, d1x, d1y, (long)blockIdx.x * blockDim.x + threadIdx.x);
-}
-
-// One RK stage (or, MODE_RHS, the right-hand side alone), one point per thread: the first oa.nblocks blocks take
-// the pure-outer points, each of the others 32 x RHS_WARPS consecutive interior points (i0 fastest), so that no lane
-// idles at the ends of rows that are no multiple of 32: 77x10x131, 8th order: 619 -> 548 us against tiles of 32 x 4
-// points, 35x2x700: 265 -> 178 us, 100x50x60: 1.24 -> 1.03 ms; rows of a multiple of 32 take the same time.
-//
-// Bound: the FP64 pipe (2 lanes a cycle per SM: 16 to 20 cycles per warp instruction), with the difference sums on the
-// integer pipe beside it (fixed_sum.cuh).  A warp does its integer passes first and its FP64 part after
-// them; four warps per scheduler (128 registers, 3 to 5 KB of spills) keep one of them in its FP64 part nearly
-// always: 640 us per right-hand side on 256x2x512, against 664 us with three (168 registers); two (255 registers, no
-// spills) were 10 % slower.  All in FP64 arithmetic, two per scheduler: 864 us.  8th order on the same grid: 1137 ->
-// 762 us; 192x96x192 spherical: 15.66 -> 10.45 ms (4th), 23.2 -> 12.9 ms (8th).
-constexpr int RHS_WARPS = 4;
-template <int FAM, int AX, int ORD>
-__global__ void __launch_bounds__(32 * RHS_WARPS, 4)
-    k_rhs(GridK G, const double* __restrict__ yin, const double* __restrict__ d1x, const double* __restrict__ d1y,
-          double* out, const double* yn, double* acc, Stage st, OuterArgs oa)
-{
-    if ((int)blockIdx.x < oa.nblocks) {
-        const int t = blockIdx.x * (32 * RHS_WARPS) + threadIdx.x;
-        if (t < oa.npts)
-            outer_point_stage<FAM, ORD, ssp_first_short<AX>()>(G, oa.pts[t], yin, out, yn, acc, oa.finf, oa.wspeed, st);
-        return;
-    }
-    const int p = (blockIdx.x - oa.nblocks) * (32 * RHS_WARPS) + threadIdx.x;
-    if (p < G.N0 * G.N1 * G.N2)
-        rhs_point_stage<FAM, AX, ORD>(G, yin, d1x, d1y, out, yn, acc, st, p % G.N0, p / G.N0);
-}
-
-// The same for grids of few points, whose time is one warp's way through its tile: a block of SPREAD_WARPS warps
-// takes 32 consecutive interior points (i0 fastest) and divides the integer passes among its warps.  64x16x2: 90
-// -> 66 us; 72x12x24: 187 -> 156 us (with k_d1 and the launches; the all-FP64 kernel took 83 and 196 us).
-// Three blocks per SM (168 registers): two are 3 % faster on the smallest grids and 35 % slower on 72x12x24, four 6
-// and 9 % slower.  It is taken up to two rounds of three blocks per SM (864 tiles: 178 against 197 us), counting the
-// tiles of every launch that runs at once; at 8,192 tiles it is half as fast as k_rhs, whose four warps share the
-// FP64 pipe (256x2x512 in 16 partitions of 512 tiles: an RK4 step of 4.71 against 3.57 ms).
-constexpr long SPREAD_TILES_PER_SM = 2 * 3;
-template <int FAM, int AX, int ORD>
-__global__ void __launch_bounds__(32 * SPREAD_WARPS, 3)
-    k_rhs_spread(GridK G, const double* __restrict__ yin, const double* __restrict__ d1x,
-                 const double* __restrict__ d1y, double* out, const double* yn, double* acc, Stage st, OuterArgs oa)
-{
-    __shared__ double tab[RawIx<AX>::N + NGF][32];
-    __shared__ int slot;
-    if ((int)blockIdx.x < oa.nblocks) {
-        const int t = blockIdx.x * (32 * SPREAD_WARPS) + threadIdx.x;
-        if (t < oa.npts)
-            outer_point_stage<FAM, ORD, ssp_first_short<AX>()>(G, oa.pts[t], yin, out, yn, acc, oa.finf, oa.wspeed, st);
-        return;
-    }
-    // the blocks of one SM put their FP64 warps on different schedulers (warp slots modulo 4)
-    if (threadIdx.x == 0) {
-        unsigned w;
-        asm volatile("mov.u32 %0, %%warpid;" : "=r"(w));
-        slot = (w / SPREAD_WARPS) % SPREAD_WARPS;
-    }
-    __syncthreads();
-    const int n = G.N0 * G.N1 * G.N2, p = (blockIdx.x - oa.nblocks) * 32 + (threadIdx.x & 31), q = p < n ? p : n - 1;
-    rhs_spread_stage<FAM, AX, ORD>(G, yin, d1x, d1y, out, yn, acc, st, q % G.N0, q / G.N0, p < n, threadIdx.x / 32,
-                                   slot, tab);
-}
-
-template <int FAM, int AX, int ORD>
-cudaError_t launch_k_rhs(cudaStream_t s, const GridK& G, const double* yin, double* d1x, double* d1y, double* out,
-                         const double* yn, double* acc, const Stage& st, const RhsLoad& load, OuterArgs oa)
-{
-    const long tiles = ((long)G.N0 * G.N1 * G.N2 + 31) / 32;
-    if (load.tiles <= SPREAD_TILES_PER_SM * load.n_sm) {
-        oa.nblocks = (oa.npts + 32 * SPREAD_WARPS - 1) / (32 * SPREAD_WARPS);
-        k_rhs_spread<FAM, AX, ORD><<<(unsigned)(tiles + oa.nblocks), 32 * SPREAD_WARPS, 0, s>>>(G, yin, d1x, d1y, out, yn,
-                                                                                              acc, st, oa);
-    } else {
-        oa.nblocks = (oa.npts + 32 * RHS_WARPS - 1) / (32 * RHS_WARPS);
-        const long nb = oa.nblocks + ((long)G.N0 * G.N1 * G.N2 + 32 * RHS_WARPS - 1) / (32 * RHS_WARPS);
-        k_rhs<FAM, AX, ORD><<<(unsigned)nb, 32 * RHS_WARPS, 0, s>>>(G, yin, d1x, d1y, out, yn, acc, st, oa);
-    }
-    return cudaGetLastError();
 }
 
 template <int FAM, int ORD>
@@ -382,12 +306,13 @@ cudaError_t launch_rhs_ord(const GridK& G, const double* yin, double* d1x, doubl
         cudaError_t e = cudaGetLastError();
         if (e != cudaSuccess) return e;
     }
+    const bool two = G.ax >= 0;
     if (G.fam == FAM_SPH) {
-        if (G.ax == 2) return launch_k_rhs<FAM_SPH, 2, ORD>(s, G, yin, d1x, d1y, out, yn, acc, st, load, oa);
-        return launch_k_rhs<FAM_SPH, -1, ORD>(s, G, yin, d1x, d1y, out, yn, acc, st, load, oa);
+        return ORD == 8 ? rhs_sph8(two, s, G, yin, d1x, d1y, out, yn, acc, st, load, oa)
+                        : rhs_sph4(two, s, G, yin, d1x, d1y, out, yn, acc, st, load, oa);
     }
-    if (G.ax == 1) return launch_k_rhs<FAM_CYL, 1, ORD>(s, G, yin, d1x, d1y, out, yn, acc, st, load, oa);
-    return launch_k_rhs<FAM_CYL, -1, ORD>(s, G, yin, d1x, d1y, out, yn, acc, st, load, oa);
+    return ORD == 8 ? rhs_cyl8(two, s, G, yin, d1x, d1y, out, yn, acc, st, load, oa)
+                    : rhs_cyl4(two, s, G, yin, d1x, d1y, out, yn, acc, st, load, oa);
 }
 
 cudaError_t launch_rhs(const GridK& G, const double* yin, double* d1x, double* d1y, double* out, const double* yn,

@@ -585,7 +585,7 @@ static int nr_part_create_body(int coords, const int Nxx[3], const nr_params* pa
                 }
             }
         // the partitions' kernels are parallel branches of the captured step
-        for (PartDev& d : s->p) s->load.add(d.K);
+        for (PartDev& d : s->p) s->load.add(d.K, d.n_outer);
         cudaError_t e = cudaDeviceGetAttribute(&s->load.n_sm, cudaDevAttrMultiProcessorCount, s->device);
         if (e == cudaSuccess) e = cudaStreamCreateWithFlags(&s->cap, cudaStreamNonBlocking);
         if (e == cudaSuccess) e = cudaEventCreateWithFlags(&s->fork, cudaEventDisableTiming);

@@ -211,10 +211,25 @@ __device__ __forceinline__ void rhs_point_stage(const GridK& G, const double* __
     stage_store<ssp_first_short<AX>()>(st, G.T, P.y - yin, k, yin, yn, out, acc);
 }
 
+constexpr int SPREAD_WARPS = 4;
+
+#ifdef __CUDACC__
+// which warp of a spread block goes on with the FP64 part: the blocks of one SM put theirs on different schedulers (warp
+// slots modulo 4); ends with the block's barrier
+__device__ __forceinline__ void spread_slot(int* slot)
+{
+    if (threadIdx.x == 0) {
+        unsigned w;
+        asm volatile("mov.u32 %0, %%warpid;" : "=r"(w));
+        *slot = (w / SPREAD_WARPS) % SPREAD_WARPS;
+    }
+    __syncthreads();
+}
+#endif
+
 // 32 interior points (point, lane by lane; lanes without one pass any valid point and active = false) by the
 // SPREAD_WARPS warps of a block: the integer-pipe passes are divided among the warps, then one warp goes on
 // with the FP64 part.  The same arithmetic as rhs_point_stage.  tab: shared memory.
-constexpr int SPREAD_WARPS = 4;
 template <int FAM, int AX, int ORD>
 __device__ __forceinline__ void rhs_spread_stage(const GridK& G, const double* __restrict__ yin,
                                                  const double* __restrict__ d1x, const double* __restrict__ d1y,

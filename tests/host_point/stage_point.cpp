@@ -164,3 +164,10 @@ extern "C" void stage_point(int coords, const int* N, const double* ampl, const 
     if (ng == 5) run<8>(coords, N, ampl, sinhw, sigma, eta, y, out, which);
     else run<4>(coords, N, ampl, sinhw, sigma, eta, y, out, which);
 }
+
+// the launch shape of the right-hand side (0, 1 spread over three or four blocks per SM; 2, 3 one point per thread, two or
+// four blocks per SM)
+extern "C" int stage_shape(int ord, int two_point, int n_sm, long tiles, long outer)
+{
+    return rhs_shape(ord, two_point != 0, RhsLoad{n_sm, tiles, outer});
+}

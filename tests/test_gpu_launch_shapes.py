@@ -1,0 +1,59 @@
+"""The launch shapes of the right-hand side (tiles spread over four warps, three or four blocks per SM; one point per
+thread, two or four blocks per SM) on sizes at the lines of the rule that chooses among them: one evaluation and
+two steps, bitwise against the same grid in a batch with a tile shape set, which always runs one point per thread.
+"""
+import numpy as np
+import pytest
+
+torch = pytest.importorskip("torch")
+
+from paper_2505_00097_gb300 import binding as B  # noqa: E402
+from paper_2505_00097_gb300 import build as BUILD  # noqa: E402
+from paper_2505_00097_gb300 import workloads as W  # noqa: E402
+
+pytestmark = pytest.mark.gpu
+
+KO8 = [0.3] * 17 + [0.99] * 7
+KINDS = {
+    "cyl_two_point": lambda n: W.sinh_cylindrical((33, 2, max(12, n // 66)), rho_max=30.0, z_max=30.0),
+    "sph_two_point": lambda n: W.sinh_spherical((33, max(10, n // 66), 2)),
+    "sph_general": lambda n: W.sinh_spherical((33, 9, 2 * max(3, n // 594))),
+    "cyl_general": lambda n: W.sinh_cylindrical((33, 6, max(12, n // 198)), rho_max=30.0, z_max=30.0),
+}
+
+
+@pytest.fixture(scope="module", autouse=True)
+def _lib():
+    if not torch.cuda.is_available():
+        pytest.skip("no CUDA device")
+    BUILD.build()
+    B.lib()
+
+
+# tiles of 32 points per SM: below and above one round of three and of four spread blocks, two rounds of three, one round
+# of two blocks of 128 points, three of them with the outer blocks on top, and more
+@pytest.mark.parametrize("per_sm", [0.2, 2.8, 3.1, 3.95, 4.3, 6.2, 8.3, 11.95, 13.0])
+@pytest.mark.parametrize("kind", sorted(KINDS))
+@pytest.mark.parametrize("order", [4, 8])
+def test_every_shape_computes_the_same_bits(order, kind, per_sm):
+    sm = torch.cuda.get_device_properties(0).multi_processor_count
+    spec = KINDS[kind](int(32 * per_sm * sm))
+    if order == 8:
+        spec = dict(spec, NG=5, ko_sigma=KO8)
+    out = []
+    for batched in (False, True):
+        g = B.Grid(spec)
+        g.set_brill_lindquist((0.6, 0.4), ((0, 0, 0.4), (0, 0, -0.6)), 1e-6, 3)
+        if batched:
+            b = B.Batch([g])
+            b.set_tile(32, 4)
+            (b.ssprk3_step if order == 8 else b.rk4_step)([g.dt_cfl], 2)
+        else:
+            (g.ssprk3_step if order == 8 else g.rk4_step)(g.dt_cfl, 2)
+        y = np.empty(24 * g.T)
+        g.get_state(y, True)
+        out.append(y)
+        if batched:
+            b.close()
+        g.close()
+    assert np.all(np.isfinite(out[0])) and np.array_equal(out[0], out[1])
