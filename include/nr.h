@@ -313,10 +313,13 @@ int nr_dt_cfl(int coords, const int Nxx[3], const nr_params* params, double* dt_
  *     on the grids' stream.  Errors: NR_EINVAL (mixed families, orders,
  *     devices, streams or azimuth kinds, duplicates), NR_ENOMEM, NR_ECUDA.
  *   nr_batch_set_tile: tile shape tile_x x tile_y of interior points per work
- *     item, one of 32x4, 64x2, 128x1, 16x8, 32x2, 64x1, 32x1 (default 16x8).
+ *     item, one of 32x4, 64x2, 128x1, 16x8, 32x2, 64x1, 32x1 (default 16x8, and
+ *     for batches of few points 32 consecutive points per item, whose difference
+ *     sums four warps share).
  *   nr_batch_autotune: times one substage launch of each compiled tile shape
- *     on the batch (it writes only the RK work buffers, not the states), keeps
- *     the fastest and returns it (synchronises).
+ *     and of the shared 32 points on the batch (it writes only the RK work
+ *     buffers, not the states), keeps the fastest and returns it, the latter as
+ *     32x1 (synchronises).
  *   nr_batch_rk4_step, nr_batch_ssprk3_step: dts[ngrids] per-grid step sizes
  *     (host), nsteps steps of RK4 or SSPRK3. */
 typedef struct nr_batch nr_batch;

@@ -40,7 +40,10 @@ struct nr_batch {
     int device = 0;
     cudaStream_t stream = nullptr;
     cudaStream_t cap = nullptr;
-    int tile = 3;             // kTiles index: 16x8, the shape the autotuner picks on the workloads
+    int tile = 3;             // kTiles index: a spread shape where rhs_shape says so, else 16x8, the shape the
+                              // autotuner picks on the workloads
+    bool few = false;         // at most two blocks of 128 points per SM (build_table)
+    int n_sm = 0;
     int total = 0;
     int total_d1 = 0;          // items of the first-difference pass
     BGrid* d_grids = nullptr;
@@ -65,8 +68,10 @@ struct DevGuard {
 int build_table(nr_batch* b, const double* dts, bool ssp)
 {
     const TileShape ts = kTiles[b->tile];
+    const int points = ts.spread ? 32 * SPREAD_WARPS : ts.tx * ts.ty;   // threads of a block
     std::vector<BGrid> h(b->grids.size());
     int w = 0;
+    long load = 0;   // threads that count for the register choice: those of the outer points only at 8th order (rhs_shape)
     for (size_t q = 0; q < b->grids.size(); q++) {
         nr_grid* g = b->grids[q];
         BGrid& B = h[q];   // value-initialised by the vector
@@ -85,9 +90,10 @@ int build_table(nr_batch* b, const double* dts, bool ssp)
         B.tiles_x = (g->K.N0 + ts.tx - 1) / ts.tx;
         const int tiles_y = (g->K.N1 * g->K.N2 + ts.ty - 1) / ts.ty;
         B.w_begin = w;
-        B.w_rhs_end = w + B.tiles_x * tiles_y;
-        B.w_end = B.w_rhs_end + (g->n_outer + ts.tx * ts.ty - 1) / (ts.tx * ts.ty);
+        B.w_rhs_end = w + (ts.spread ? (g->K.N0 * g->K.N1 * g->K.N2 + 31) / 32 : B.tiles_x * tiles_y);
+        B.w_end = B.w_rhs_end + (g->n_outer + points - 1) / points;
         w = B.w_end;
+        load += (long)points * ((b->ord == 8 ? B.w_end : B.w_rhs_end) - B.w_begin);
         // the same stage constants as the single-grid drivers
         const double dt = dts[q];
         const int enf = g->P.enforce_detgb;
@@ -104,6 +110,7 @@ int build_table(nr_batch* b, const double* dts, bool ssp)
         }
     }
     b->total = w;
+    b->few = load <= 2L * 128 * b->n_sm;
     int w1 = 0;
     for (size_t q = 0; q < b->grids.size(); q++) {
         h[q].d1_begin = w1;
@@ -132,10 +139,10 @@ cudaError_t enqueue_stage_launch(nr_batch* b, int stage, cudaStream_t s)
                         : batch_d1_cyl4(tp, b->d_grids, n, b->total_d1, stage, s);
     if (e != cudaSuccess) return e;
     if (b->fam == FAM_SPH)
-        return b->ord == 8 ? batch_stage_sph8(tp, b->tile, b->d_grids, n, b->total, stage, s)
-                           : batch_stage_sph4(tp, b->tile, b->d_grids, n, b->total, stage, s);
-    return b->ord == 8 ? batch_stage_cyl8(tp, b->tile, b->d_grids, n, b->total, stage, s)
-                       : batch_stage_cyl4(tp, b->tile, b->d_grids, n, b->total, stage, s);
+        return b->ord == 8 ? batch_stage_sph8(tp, b->tile, b->few, b->d_grids, n, b->total, stage, s)
+                           : batch_stage_sph4(tp, b->tile, b->few, b->d_grids, n, b->total, stage, s);
+    return b->ord == 8 ? batch_stage_cyl8(tp, b->tile, b->few, b->d_grids, n, b->total, stage, s)
+                       : batch_stage_cyl4(tp, b->tile, b->few, b->d_grids, n, b->total, stage, s);
 }
 
 // one step of the table's integrator; every stage copies the ghosts the stencils read (the
@@ -247,6 +254,12 @@ static int nr_batch_create_body(nr_grid* const* grids, int ngrids, nr_batch** ou
             }
         }
         b->n_inner_stencil = (int)inner.size();
+        RhsLoad load;
+        load.n_sm = b->n_sm = grids[0]->load.n_sm;
+        for (int q = 0; q < ngrids; q++) load.add(grids[q]->K, grids[q]->n_outer);
+        const RhsShape shape = rhs_shape(b->fam, b->ord, b->two_point, load);
+        if (shape == RHS_SPREAD3) b->tile = kNumTiles;
+        if (shape == RHS_SPREAD4) b->tile = kNumTiles + 1;
         cudaError_t e = cudaMalloc(&b->d_grids, sizeof(BGrid) * ngrids);
         if (e == cudaSuccess) e = cudaMalloc(&b->d_inner, sizeof(BInner) * std::max<size_t>(inner.size(), 1));
         if (e == cudaSuccess && !inner.empty())
@@ -306,7 +319,7 @@ static int nr_batch_autotune_body(nr_batch* b, const double* dts, int* tile_x, i
     int best = -1;
     float best_t = 1e30f;
     int rc = NR_OK;
-    for (int t = 0; t < kNumTiles && rc == NR_OK; t++) {
+    for (int t = 0; t < kNumShapes && rc == NR_OK; t++) {
         b->tile = t;
         if ((rc = build_table(b, dts, b->table_ssp))) break;
         // stage 1 writes only the stage buffer and the accumulator: the state is untouched

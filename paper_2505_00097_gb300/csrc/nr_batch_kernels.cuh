@@ -2,9 +2,9 @@
 // launch helpers, instantiated once per coordinate family and finite-difference
 // order (nr_batch_{sph,cyl}{,8}.cu) so the four compile in parallel.
 //
-// A work item is either a tx x ty tile of one grid's interior points or a chunk of tx * ty of its
-// pure-outer ghost points.  One launch per RK substage covers the items of all grids, one block of
-// tx * ty threads per item: the block finds its grid
+// A work item is a tx x ty tile of one grid's interior points, or, in the spread shapes of small batches, 32
+// consecutive ones, or a chunk of its pure-outer ghost points.  One launch per RK substage covers the items of all
+// grids, one block per item (tx * ty threads; spread: four warps, as k_rhs_spread): the block finds its grid
 // by binary search over the items' start indices and stages that grid's
 // record in shared memory.  Every
 // point runs the same per-point code as the single-grid kernels
@@ -28,13 +28,13 @@ struct __align__(16) BGrid {
     const double* finf;
     const double* wspeed;
     int n_outer;
-    int tiles_x, tx;           // tiles of tx columns, blockDim.x points
+    int tiles_x, tx;           // tiles of tx columns, blockDim.x points (not in the spread shapes)
     int w_begin, w_rhs_end, w_end;
     int ssp;                   // the table's integrator: 0 RK4 (st[0..3]), 1 SSPRK3 (st[0..2])
     Stage st[4];
 };
 
-constexpr int BATCH_MAX_THREADS = 128, BATCH_MIN_BLOCKS = 4;
+constexpr int BATCH_MAX_THREADS = 128;
 
 struct BInner {
     int grid, dst, src, negmask;
@@ -53,27 +53,34 @@ __device__ __forceinline__ void stage_buffers(const BGrid& B, int stage, const d
     }
 }
 
-template <int FAM, int AX, int ORD>
-__global__ void __launch_bounds__(BATCH_MAX_THREADS, BATCH_MIN_BLOCKS) k_batch_stage(const BGrid* __restrict__ grids,
-                                                                                      int ngrids, int total, int stage)
+// the grid of work item w, its record staged in shared memory; ends with the block's barrier
+__device__ __forceinline__ const BGrid& batch_grid(const BGrid* __restrict__ grids, int ngrids, int w,
+                                                   unsigned long long* s_grid)
 {
-    // one block per work item; the item's grid record is staged in shared memory
-    __shared__ __align__(16) unsigned long long s_grid[(sizeof(BGrid) + 7) / 8];
-    const int tid = threadIdx.x;
-    const int w = (int)blockIdx.x;
-    if (w >= total) return;
     int lo = 0, hi = ngrids - 1;
     while (lo < hi) {
         const int mid = (lo + hi + 1) >> 1;
         if (grids[mid].w_begin <= w) lo = mid;
         else hi = mid - 1;
     }
-    {
-        const unsigned long long* src = reinterpret_cast<const unsigned long long*>(grids + lo);
-        for (int q = tid; q < (int)(sizeof(BGrid) / 8); q += blockDim.x) s_grid[q] = src[q];
-    }
+    const unsigned long long* src = reinterpret_cast<const unsigned long long*>(grids + lo);
+    for (int q = threadIdx.x; q < (int)(sizeof(BGrid) / 8); q += blockDim.x) s_grid[q] = src[q];
     __syncthreads();
-    const BGrid& B = *reinterpret_cast<const BGrid*>(s_grid);
+    return *reinterpret_cast<const BGrid*>(s_grid);
+}
+constexpr int BGRID_WORDS = (sizeof(BGrid) + 7) / 8;
+
+// one block per work item; BPS blocks of BATCH_MAX_THREADS per SM (registers), two in batches that leave no scheduler more
+// than two warps (rhs_shape), as k_rhs
+template <int FAM, int AX, int ORD, int BPS>
+__global__ void __launch_bounds__(BATCH_MAX_THREADS, BPS) k_batch_stage(const BGrid* __restrict__ grids, int ngrids,
+                                                                        int total, int stage)
+{
+    __shared__ __align__(16) unsigned long long s_grid[BGRID_WORDS];
+    const int tid = threadIdx.x;
+    const int w = (int)blockIdx.x;
+    if (w >= total) return;
+    const BGrid& B = batch_grid(grids, ngrids, w, s_grid);
     const double* yin;
     const double* yn;
     double* out;
@@ -90,6 +97,35 @@ __global__ void __launch_bounds__(BATCH_MAX_THREADS, BATCH_MIN_BLOCKS) k_batch_s
             outer_point_stage<FAM, ORD, ssp_first_short<AX>()>(B.K, B.outer[p], yin, out, yn, B.acc, B.finf, B.wspeed,
                                                                B.st[stage]);
     }
+}
+
+// The same for batches of few points (rhs_shape), 32 consecutive points per block of four warps, as k_rhs_spread.  Per RK
+// step: six 64x16x2 grids 382 -> 296 us (all-FP64: 341)
+template <int FAM, int AX, int ORD, int BPS>
+__global__ void __launch_bounds__(32 * SPREAD_WARPS, BPS) k_batch_spread(const BGrid* __restrict__ grids, int ngrids,
+                                                                         int total, int stage)
+{
+    __shared__ __align__(16) unsigned long long s_grid[BGRID_WORDS];
+    __shared__ double tab[RawIx<AX>::N + NGF][32];
+    __shared__ int slot;
+    const int w = (int)blockIdx.x;
+    if (w >= total) return;
+    const BGrid& B = batch_grid(grids, ngrids, w, s_grid);
+    const double* yin;
+    const double* yn;
+    double* out;
+    stage_buffers(B, stage, yin, out, yn);
+    if (w >= B.w_rhs_end) {
+        const int p = (w - B.w_rhs_end) * (32 * SPREAD_WARPS) + threadIdx.x;
+        if (p < B.n_outer)
+            outer_point_stage<FAM, ORD, ssp_first_short<AX>()>(B.K, B.outer[p], yin, out, yn, B.acc, B.finf, B.wspeed,
+                                                               B.st[stage]);
+        return;
+    }
+    spread_slot(&slot);
+    const int n = B.K.N0 * B.K.N1 * B.K.N2, p = (w - B.w_begin) * 32 + (threadIdx.x & 31), q = p < n ? p : n - 1;
+    rhs_spread_stage<FAM, AX, ORD>(B.K, yin, B.d1x, B.d1y, out, yn, B.acc, B.st[stage], q % B.K.N0, q / B.K.N0, p < n,
+                                   threadIdx.x / 32, slot, tab);
 }
 
 // the stored first differences of every grid's stage input, 256 points per block
@@ -112,17 +148,25 @@ __global__ void __launch_bounds__(256) k_batch_d1(const BGrid* __restrict__ grid
     d1_point<AX, ORD>(B.K, yin, B.d1x, B.d1y, (long)(w - B.d1_begin) * 256 + threadIdx.x);
 }
 
-// tile shapes the autotuner tries
+// work-item shapes the autotuner tries: tiles, which nr_batch_set_tile can ask for too, and 32 points spread over four
+// warps with three or four blocks per SM
 struct TileShape {
-    int tx, ty;
+    int tx, ty, spread;
 };
-constexpr TileShape kTiles[] = {{32, 4}, {64, 2}, {128, 1}, {16, 8}, {32, 2}, {64, 1}, {32, 1}};
-constexpr int kNumTiles = sizeof(kTiles) / sizeof(kTiles[0]);
+constexpr TileShape kTiles[] = {{32, 4, 0}, {64, 2, 0}, {128, 1, 0}, {16, 8, 0}, {32, 2, 0},
+                                {64, 1, 0}, {32, 1, 0}, {32, 1, 3},  {32, 1, 4}};
+constexpr int kNumShapes = sizeof(kTiles) / sizeof(kTiles[0]), kNumTiles = kNumShapes - 2;
 
+// few: the batch is small enough for two blocks per SM
 template <int FAM, int AX, int ORD>
-cudaError_t launch_bstage(int tile, const BGrid* g, int n, int total, int stage, cudaStream_t s)
+cudaError_t launch_bstage(int tile, bool few, const BGrid* g, int n, int total, int stage, cudaStream_t s)
 {
-    if (total > 0) k_batch_stage<FAM, AX, ORD><<<total, kTiles[tile].tx * kTiles[tile].ty, 0, s>>>(g, n, total, stage);
+    const TileShape t = kTiles[tile];
+    if (total <= 0) return cudaSuccess;
+    if (t.spread == 3) k_batch_spread<FAM, AX, ORD, 3><<<total, 32 * SPREAD_WARPS, 0, s>>>(g, n, total, stage);
+    else if (t.spread == 4) k_batch_spread<FAM, AX, ORD, 4><<<total, 32 * SPREAD_WARPS, 0, s>>>(g, n, total, stage);
+    else if (few) k_batch_stage<FAM, AX, ORD, 2><<<total, t.tx * t.ty, 0, s>>>(g, n, total, stage);
+    else k_batch_stage<FAM, AX, ORD, 4><<<total, t.tx * t.ty, 0, s>>>(g, n, total, stage);
     return cudaGetLastError();
 }
 
@@ -137,8 +181,8 @@ cudaError_t launch_batch_d1(const BGrid* g, int n, int total_d1, int stage, cuda
 // NRK_BATCH_LAUNCH, the substage launch (tile shape `tile`) and the first-difference pass
 // of all grids; two_point: the grids' azimuth holds two points (GridK::ax >= 0)
 #define NRK_BATCH_DECL(NAME)                                                                                   \
-    cudaError_t batch_stage_##NAME(bool two_point, int tile, const BGrid* g, int n, int total, int stage,      \
-                                   cudaStream_t s);                                                            \
+    cudaError_t batch_stage_##NAME(bool two_point, int tile, bool few, const BGrid* g, int n, int total,       \
+                                   int stage, cudaStream_t s);                                                 \
     cudaError_t batch_d1_##NAME(bool two_point, const BGrid* g, int n, int total_d1, int stage, cudaStream_t s);
 NRK_BATCH_DECL(sph4)
 NRK_BATCH_DECL(sph8)
@@ -146,11 +190,11 @@ NRK_BATCH_DECL(cyl4)
 NRK_BATCH_DECL(cyl8)
 
 #define NRK_BATCH_LAUNCH(NAME, FAM_, AXTWO_, ORD_)                                                             \
-    cudaError_t batch_stage_##NAME(bool two_point, int tile, const BGrid* g, int n, int total, int stage,      \
-                                   cudaStream_t s)                                                             \
+    cudaError_t batch_stage_##NAME(bool two_point, int tile, bool few, const BGrid* g, int n, int total,       \
+                                   int stage, cudaStream_t s)                                                  \
     {                                                                                                          \
-        return two_point ? launch_bstage<FAM_, AXTWO_, ORD_>(tile, g, n, total, stage, s)                      \
-                         : launch_bstage<FAM_, -1, ORD_>(tile, g, n, total, stage, s);                         \
+        return two_point ? launch_bstage<FAM_, AXTWO_, ORD_>(tile, few, g, n, total, stage, s)                 \
+                         : launch_bstage<FAM_, -1, ORD_>(tile, few, g, n, total, stage, s);                    \
     }                                                                                                          \
     cudaError_t batch_d1_##NAME(bool two_point, const BGrid* g, int n, int total_d1, int stage, cudaStream_t s) \
     {                                                                                                          \

@@ -102,7 +102,10 @@ struct RhsLoad {
 // about as long as its fullest SM, so the lines lie where a round is full, counted in the device's SMs.  us per RK step on
 // a GB300 (152 SMs) beside the other shapes, and beside the all-FP64 kernel of one point per thread; cyl2 = 64x2xN,
 // cyl = 64x8xN cylindrical, sph2 = 64xNx2, sph = 64x16xN spherical:
-//   one round of three spread blocks: cyl2, 304 tiles: 264, four 274, points 326 (two) and 352 (four), all-FP64 318
+//   one round of three spread blocks: cyl2, 304 tiles: 264, four 274, points 326 (two) and 352 (four), all-FP64 318;
+//     of two with cylindrical coordinates, two-point azimuth and 8th order, whose outer blocks (two one-sided 9-point
+//     sums) take spread blocks' slots: cyl2, 400: 311, points 301, all-FP64 300; three grids of 35x2x50 and more: 341, 317,
+//     302 (sph2, 400: 281, 320, 321)
 //   one round of four: cyl2, 520 tiles: 311, three 462, points 327 and 352, all-FP64 319; sph, 576: 423, 653, 464, 531, 443.
 //     Not with two-point azimuth and 8th order, where the integer part outweighs the FP64 part: cyl2, 520: points 295,
 //     four 354, all-FP64 301; sph2, 520: 319, 342, 326
@@ -112,10 +115,10 @@ struct RhsLoad {
 //     the 8th order are as long as tiles and count: cyl2, 1184, 8th: 719, four 657
 //   outer blocks alone would put a fourth block on an SM, 4th order: cyl2, 1824: 811, four 925, all-FP64 902
 enum RhsShape { RHS_SPREAD3, RHS_SPREAD4, RHS_POINTS2, RHS_POINTS4 };
-inline RhsShape rhs_shape(int ord, bool two_point, const RhsLoad& l)
+inline RhsShape rhs_shape(int fam, int ord, bool two_point, const RhsLoad& l)
 {
     const long sm = l.n_sm, all = l.tiles + l.outer, blocks = (l.tiles + 3) / 4;
-    if (all <= 3 * sm) return RHS_SPREAD3;
+    if (all <= (fam == 1 && two_point && ord == 8 ? 2 : 3) * sm) return RHS_SPREAD3;   // 1: FAM_CYL
     if (all <= 4 * sm && !(two_point && ord == 8)) return RHS_SPREAD4;
     if (l.tiles > 4 * sm && all <= 6 * sm) return RHS_SPREAD3;
     if (blocks + (ord == 8 ? l.outer : 0) <= 2 * sm) return RHS_POINTS2;

@@ -71,7 +71,7 @@ cudaError_t launch_k_rhs(cudaStream_t s, const GridK& G, const double* yin, doub
     oa.nblocks = (oa.npts + 32 * RHS_WARPS - 1) / (32 * RHS_WARPS);
     const long n = (long)G.N0 * G.N1 * G.N2, tiles = (n + 31) / 32, blocks = (n + 32 * RHS_WARPS - 1) / (32 * RHS_WARPS);
     const unsigned ng = (unsigned)(blocks + oa.nblocks), ns = (unsigned)(tiles + oa.nblocks);
-    switch (rhs_shape(G.ord, G.ax >= 0, load)) {
+    switch (rhs_shape(FAM, ORD, AX >= 0, load)) {
     case RHS_SPREAD3: k_rhs_spread<FAM, AX, ORD, 3><<<ns, 32 * SPREAD_WARPS, 0, s>>>(G, yin, d1x, d1y, out, yn, acc, st, oa); break;
     case RHS_SPREAD4: k_rhs_spread<FAM, AX, ORD, 4><<<ns, 32 * SPREAD_WARPS, 0, s>>>(G, yin, d1x, d1y, out, yn, acc, st, oa); break;
     case RHS_POINTS2: k_rhs<FAM, AX, ORD, 2><<<ng, 32 * RHS_WARPS, 0, s>>>(G, yin, d1x, d1y, out, yn, acc, st, oa); break;

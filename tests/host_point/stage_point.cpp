@@ -167,7 +167,7 @@ extern "C" void stage_point(int coords, const int* N, const double* ampl, const 
 
 // the launch shape of the right-hand side (0, 1 spread over three or four blocks per SM; 2, 3 one point per thread, two or
 // four blocks per SM)
-extern "C" int stage_shape(int ord, int two_point, int n_sm, long tiles, long outer)
+extern "C" int stage_shape(int fam, int ord, int two_point, int n_sm, long tiles, long outer)
 {
-    return rhs_shape(ord, two_point != 0, RhsLoad{n_sm, tiles, outer});
+    return rhs_shape(fam, ord, two_point != 0, RhsLoad{n_sm, tiles, outer});
 }

@@ -57,3 +57,40 @@ def test_every_shape_computes_the_same_bits(order, kind, per_sm):
             b.close()
         g.close()
     assert np.all(np.isfinite(out[0])) and np.array_equal(out[0], out[1])
+
+
+# grids of uneven sizes, tiles per SM of the whole batch: one round of three and of four spread blocks, two rounds of
+# three, one point per thread with two and with four blocks per SM
+@pytest.mark.parametrize("choice", ["default", "autotune"])
+@pytest.mark.parametrize("per_sm", [0.5, 3.6, 5.2, 7.0, 13.0])
+@pytest.mark.parametrize("kind", sorted(KINDS))
+@pytest.mark.parametrize("order", [4, 8])
+def test_a_batch_of_any_shape_computes_the_bits_of_its_grids(order, kind, per_sm, choice):
+    sm = torch.cuda.get_device_properties(0).multi_processor_count
+    specs = [KINDS[kind](int(32 * per_sm * sm * w)) for w in (0.2, 0.5, 0.3)]
+    if order == 8:
+        specs = [dict(s, NG=5, ko_sigma=KO8) for s in specs]
+    out = []
+    for batched in (False, True):
+        grids = [B.Grid(s) for s in specs]
+        for q, g in enumerate(grids):
+            g.set_brill_lindquist((0.6, 0.4), ((0, 0, 0.4), (0, 0, -0.6)), 1e-6, 3 + q)
+        dts = [g.dt_cfl for g in grids]
+        if batched:
+            b = B.Batch(grids)
+            if choice == "autotune":
+                b.autotune(dts)
+            (b.ssprk3_step if order == 8 else b.rk4_step)(dts, 2)
+        else:
+            for g, dt in zip(grids, dts):
+                (g.ssprk3_step if order == 8 else g.rk4_step)(dt, 2)
+        for g in grids:
+            y = np.empty(24 * g.T)
+            g.get_state(y, True)
+            out.append(y)
+        if batched:
+            b.close()
+        for g in grids:
+            g.close()
+    for a, c in zip(out[:3], out[3:]):
+        assert np.all(np.isfinite(a)) and np.array_equal(a, c)
