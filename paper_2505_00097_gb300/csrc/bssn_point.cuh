@@ -1395,10 +1395,8 @@ __device__ __forceinline__ void fx_upko(const fx_i64* v, fx_i64& U, fx_i64& K)
         for (int o = -G; o <= G; o++)
             if (F::up(o)) U += F::up(o) * v[G + o];
     } else {
-        // 64-bit values times up to 11 bits of weight, summed in a high and a low word (which starts at half of what
-        // the shift drops: the sums are rounded, not cut)
-        constexpr fx_i64 half = 1LL << (F::Q - 1);
-        fx_i64 uh = 0, ul = half;
+        // 64-bit values times up to 11 bits of weight, summed in a high and a low word
+        fx_i64 uh = 0, ul = 0;
 #pragma unroll
         for (int o = -G; o <= G; o++)
             if (F::up(o)) {
@@ -1407,15 +1405,15 @@ __device__ __forceinline__ void fx_upko(const fx_i64* v, fx_i64& U, fx_i64& K)
                 ul += (fx_i64)s.l * F::up(o);
             }
         const FxSplit c = fx_split(v[G]);
-        fx_i64 kh = (fx_i64)c.h * F::ko(0), kl = (fx_i64)c.l * F::ko(0) + half;
+        fx_i64 kh = (fx_i64)c.h * F::ko(0), kl = (fx_i64)c.l * F::ko(0);
 #pragma unroll
         for (int o = 1; o <= G; o++) {
             const FxSplit s = fx_split(v[G + o] + v[G - o]);
             kh += (fx_i64)s.h * F::ko(o);
             kl += (fx_i64)s.l * F::ko(o);
         }
-        U = (uh << (32 - F::Q)) + (ul >> F::Q);
-        K = (kh << (32 - F::Q)) + (kl >> F::Q);
+        U = fx_shift<F::Q>(uh, ul);
+        K = fx_shift<F::Q>(kh, kl);
     }
 }
 
@@ -1538,8 +1536,8 @@ __device__ __forceinline__ void adv_ko_sums(const double* y, long T, const long 
                 const FxSplit kap = g < G_VET ? ck[0][d] : ck[1][d];
                 if (d == AX) {
                     const fx_i64 w = fx_in<F::SH>(in.o, E) - vc;
-                    fx_mac(dot, kap, fx_split(F::a_log2 >= F::Q ? w << (F::a_log2 >= F::Q ? F::a_log2 - F::Q : 0)
-                                                                : w >> (F::Q >= F::a_log2 ? F::Q - F::a_log2 : 0)));
+                    if constexpr (F::a_log2 >= F::Q) fx_mac(dot, kap, fx_split(w << (F::a_log2 - F::Q)));
+                    else fx_mac(dot, kap, fx_split(fx_shift<F::Q - F::a_log2>(w)));
                     continue;
                 }
                 fx_i64 v[2 * G + 1], U, K;

@@ -80,6 +80,17 @@ __device__ __forceinline__ void fx_mac(FxDot& d, FxSplit a, FxSplit b)
     d.cross += fx_mulhi(a.l, b.l);
 }
 
+// x / 2^Q and (h 2^32 + l) / 2^Q rounded to nearest, ties away from zero: the same for either sign, so that a sum of
+// negated values is the negated sum (a field and its mirror image stay mirror images)
+template <int Q>
+__device__ __forceinline__ fx_i64 fx_shift(fx_i64 x) { return (x + (1LL << (Q - 1)) + (x >> 63)) >> Q; }
+template <int Q>
+__device__ __forceinline__ fx_i64 fx_shift(fx_i64 h, fx_i64 l)
+{
+    const fx_i64 t = h + (l >> 32);
+    return (t << (32 - Q)) + ((fx_i64)((fx_u64)(unsigned)l + (1ULL << (Q - 1)) + (fx_u64)(t >> 63)) >> Q);
+}
+
 __device__ __forceinline__ int fx_clz(fx_u64 a) { return __clzll((fx_i64)a); }   // 64 for 0
 
 // a 2^e (a = 1.x 2^63, or 0) with sign s (0 or -1) as an FP64 number, rounded to nearest

@@ -137,3 +137,21 @@ def test_advection_and_dissipation_at_the_top_of_a_binade(lib, order, ax):
         c = max(Fr(float(abs(vet[0]) * D[0])), Fr(float(float(KC[order]) * sigma * D[0])))
         bound = abs(tot) / 2 ** 53 + c * Fr(float(x)) * (weights * (Fr(1, 2 ** (52 + sh)) + Fr(1, 2 ** 58)) + last)
         assert abs(Fr(float(out[0])) - tot) <= bound, (x, follow, flip, vs, kap, out[0], float(tot))
+
+
+@pytest.mark.parametrize("ax", [-1, 1, 2])
+@pytest.mark.parametrize("order", [4, 8])
+def test_negated_values_give_the_negated_sum(lib, order, ax):
+    """Smooth fields: the bits of the sum with its sign flipped, so that a state with a reflection symmetry keeps it."""
+    rng = np.random.default_rng(17 + order + ax)
+    x = np.arange(11) - 5
+    for _ in range(400):
+        k, p = rng.uniform(0.02, 0.2, 3), rng.uniform(0, 6, 3)
+        f = rng.uniform(-1, 1) + np.zeros((11, 11, 11))
+        for d in range(3):
+            f += np.cos(k[d] * x + p[d]).reshape([11 if 2 - i == d else 1 for i in range(3)])
+        vet, D = rng.uniform(-0.1, 0.1, 3), 10.0 ** rng.uniform(-1, 1, 3)
+        out = [np.empty(1), np.empty(1)]
+        for o, s in zip(out, (1.0, -1.0)):
+            lib.fixed_advko(ax, order, _p(np.ascontiguousarray(s * f)), _p(vet), _p(D), ctypes.c_double(0.3), _p(o), _p(np.empty(1)))
+        assert out[0][0] == -out[1][0]
