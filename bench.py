@@ -51,33 +51,44 @@ from paper_2505_00097_gb300 import workloads as W  # noqa: E402
 METRIC = "BSSN FP64 point-updates/s (RK4 substeps)"
 UNIT = "point-updates/s"
 
-# FP64 operations (FMA = 2) per interior point of one RHS evaluation (nr_rhs:
-# the k_d1 pre-pass and k_rhs), by workload (the kernel variant it runs): the FP64 operations of the algorithm
-# as the point code's source has them (add + mul + div + 2 fma, a host census that a test recomputes), with
-# the raw first differences counted as FP64 sums.  The kernels take those, and the advection + dissipation sums
-# (not counted here at all), in integer arithmetic beside the FP64 pipe.
+# FP64 operations (FMA = 2) per interior point of one RHS evaluation (nr_rhs: the k_d1 pre-pass and k_rhs) that the
+# compiled kernels issue, by workload (the kernel variant it runs): (DADD + DMUL + 2 DFMA) / interior points in one
+# ncu capture of that workload's nr_rhs.  This is the work of the FP64 pipe; the advection + dissipation sums and
+# most first and mixed differences run on the integer pipe and are not in it.  Head-on 256x2x512: k_rhs 162 / 294 / 701,
+# k_d1 10.1 / 0 / 5.0; 8th order: 210 / 315 / 748, 20.3 / 5.1 / 15.2.  Large 3D, counted on 96x48x96: k_rhs 228 / 375 / 993
+# and 293 / 409 / 1059; k_d1 takes five of eleven differences in FP64, 3 instructions (4 FLOP) or 8 (11) each, for
+# 22.46 and 22.93 stored differences per point at 384x192x384.
+F_PIPE = {"headon": 1878.2, "headon8": 2076.9, "large3d": 2629.8, "large3d8": 2934.7}
+# F_PIPE over twice those instructions: the fraction of the FLOP peak that a fully busy FP64 pipe reaches with this mix (a
+# DADD or DMUL takes an FMA's issue slot for 1 FLOP)
+PIPE_CEILING = {"headon": 0.8012, "headon8": 0.7905, "large3d": 0.8084, "large3d8": 0.7956}
+# The operations of the algorithm as the point code's source has them (add + mul + div + 2 fma, a host census that a
+# test recomputes), with the first and mixed differences counted as FP64 sums and the advection + dissipation
+# sums not counted: a rate of useful work, part of which is not the FP64 pipe's
 F_ALG = {"headon": 2071.3, "large3d": 2963.8, "headon8": 2513.9, "large3d8": 3749.2}
-# DRAM bytes (read + write) of the k_d1 and k_rhs launches of one nr_rhs in an ncu capture; for the large 3D grids the
-# capture's bytes per interior point at 96x48x96 (6144.5 and 6816.1, mostly register-spill lines)
-# times the 28,311,552 points of the full grid
-TRAFFIC = {"headon": 24019200 + 80128 + 304581120 + 714723072,
-           "headon8": 24950016 + 105216 + 334224896 + 801484032,
-           "large3d": round(6144.5 * 28311552), "large3d8": round(6816.1 * 28311552)}
-# The same without the k_d1 pre-pass
+# the same without the k_d1 pre-pass
 KERNEL_CENSUS = {"headon": 2027, "headon8": 2391, "large3d": 2874, "large3d8": 3497}
-# FLOPs over twice the FP64 instructions of the same source (k_d1 + k_rhs): the fraction of the FLOP peak
-# that a fully busy FP64 pipe reaches with this mix (a DADD or DMUL takes an FMA's issue slot for 1 FLOP)
+# F_ALG over twice its operations (k_d1 + k_rhs)
 MIX_CEILING = {"headon": 0.7827, "headon8": 0.7667, "large3d": 0.7923, "large3d8": 0.7710}
+# DRAM bytes (read + write) of the k_d1 and k_rhs launches of one nr_rhs in that capture; for the large 3D grids the
+# capture's bytes per interior point at 96x48x96 (6208.0 and 6770.5, mostly register-spill lines)
+# times the 28,311,552 points of the full grid
+TRAFFIC = {"headon": 24031744 + 87040 + 307848704 + 731901184,
+           "headon8": 24973824 + 117248 + 328414464 + 809833216,
+           "large3d": round(6208.0 * 28311552), "large3d8": round(6770.5 * 28311552)}
 # FP64 operations (add + mul + div) per interior point of one RHS evaluation as the oracle's counting
 # build counts them: the plain coordinate-basis evaluation of the same discretisation with generic index
 # loops and the reference metric evaluated at every point -- the work of the method evaluated plainly.
 # Achieved against it (frac_method) can exceed 1: the kernels compute the same discrete right-hand side
 # with about a tenth of those operations
 F_METHOD = {"headon": 28967, "headon8": 49631, "large3d": 28970, "large3d8": 49634}
-# The same for the diagnostics, per interior point of one call, by workload: the constraints' FP64 operations as the
-# point code's source has them (a host census that a test recomputes: FMA = 2, one division, the square root of |M| not
-# counted; their first and mixed differences counted as FP64 sums, which the kernels take on the integer pipe), psi4's
-# from an ncu capture of k_psi4 (460 / 434 / 1016 DADD / DMUL / DFMA); absent: not counted
+# The diagnostics per interior point of one call, by workload: what the FP64 pipe executes, from an ncu capture of those
+# kernels on the head-on state (k_ham 100 / 214 / 458 DADD / DMUL / DFMA, k_mom 26 / 144 / 220, k_psi4 460 / 434 / 1016);
+# absent: not captured
+DIAG_PIPE = {"headon": {"hamiltonian": 1230.0, "momentum": 610.0, "psi4": 2926.0}}
+# the operations of the algorithm: the constraints' point code by a host census that a test recomputes (FMA = 2, one
+# division, the square root of |M| not counted; their first and mixed differences counted as FP64 sums, which the
+# kernels take on the integer pipe), psi4 as captured
 DIAG_FLOPS = {"headon": {"hamiltonian": 1767.0, "momentum": 737.0, "psi4": 2926.0}}
 # the census alone
 DIAG_CENSUS = {"headon": {"hamiltonian": 1767, "momentum": 737}}
@@ -460,13 +471,18 @@ def run_ours(args, spec, world, rank, local):
             "traffic": TRAFFIC.get(args.workload), "traffic_algorithmic": B_ALG_RHS * pts,
             "traffic_source": "ncu dram__bytes_read.sum + dram__bytes_write.sum of one nr_rhs (k_d1 + k_rhs); "
                               "the excess over the algorithmic bytes is register-spill lines evicted to DRAM"}
-    f_alg = F_ALG.get(args.workload)
-    if f_alg:
-        ach = f_alg * pts / (rhs_ms * 1e-3)
-        roof.update(achieved=ach / 1e12, frac=ach / peak, flops_per_point=f_alg,
-                    flops_source="FP64 operations per interior point in the kernels' source (host census); the "
-                                 "advection + dissipation sums run on the integer pipe and are not counted",
-                    mix_ceiling=MIX_CEILING[args.workload])
+    f_pipe = F_PIPE.get(args.workload)
+    if f_pipe:
+        f_alg = F_ALG[args.workload]
+        ach = f_pipe * pts / (rhs_ms * 1e-3)
+        roof.update(achieved=ach / 1e12, frac=ach / peak, flops_per_point=f_pipe,
+                    flops_source="the compiled kernels' DADD + DMUL + 2 DFMA per interior point (ncu); the advection + "
+                                 "dissipation sums and most first and mixed differences run on the integer pipe and "
+                                 "are not counted",
+                    mix_ceiling=PIPE_CEILING[args.workload], flops_per_point_algorithm=f_alg,
+                    achieved_algorithm=f_alg * pts / (rhs_ms * 1e-3) / 1e12,
+                    algorithm_source="FP64 operations per interior point in the kernels' source (host census), the "
+                                     "first and mixed differences counted as FP64 sums")
     else:
         roof.update(achieved=None, frac=None, flops_per_point=None)
     f_method = F_METHOD.get(args.workload)
@@ -593,9 +609,10 @@ def diagnostics(g, spec, stream, wl: str, nrep: int) -> dict:
         torch.cuda.synchronize()
         ms = e0.elapsed_time(e1) / nrep
         d = {"launches": what, "device_ms": ms, "points_per_s": pts / (ms * 1e-3)}
-        f = DIAG_FLOPS.get(wl, {}).get(name)
+        f = DIAG_PIPE.get(wl, {}).get(name)
         if f:
-            d.update(flops_per_point=f, achieved_tflops=f * pts / (ms * 1e-3) / 1e12)
+            d.update(flops_per_point=f, achieved_tflops=f * pts / (ms * 1e-3) / 1e12,
+                     flops_per_point_algorithm=DIAG_FLOPS[wl][name])
         out[name] = d
     R = spec.get("psi4_radius")
     if R:
