@@ -205,8 +205,8 @@ __host__ __device__ constexpr bool ddbz(int kl, int i)
 // Gridfunctions with second derivatives (h, W, alpha, vet) have their raw first
 // differences along axis 0 (and, for a general grid, axis 1) stored by a
 // pre-pass (k_d1).  A mixed second difference is the first difference of
-// those along the other axis -- the same expression mixraw evaluates -- so the
-// stored path gives bitwise the result of the inline one.
+// those along the other axis.  Stored as FP64 sums they give bitwise what mixraw gives; k_d1 takes six of the eleven
+// gridfunctions, and the kernels all mixed differences, on the integer pipe, which rounds each difference once.
 constexpr int N_D1 = 11;
 __host__ __device__ constexpr int d1slot(int gf)
 {
@@ -215,9 +215,11 @@ __host__ __device__ constexpr int d1slot(int gf)
 __host__ __device__ constexpr int d1gf(int q) { return q < 6 ? q : q == 6 ? G_CF : q == 7 ? G_ALPHA : G_VET + q - 8; }
 
 // Where the raw difference sums of a point come from (template parameter S): differenced inline from the
-// state (0); the mixed differences, and the first differences of the same gridfunctions along axes 0 and 1, from
-// the stored first differences (1); the same with every further first difference, of the state and of the
-// stored differences, taken beforehand on the integer pipe and read from a table (2, 3).  The second
+// state (0: psi4, the allocation-free Hamiltonian constraint and host checks); the mixed differences, and the
+// first differences of the same gridfunctions along axes 0 and 1, from the stored first differences (1: host checks and
+// the host census, which counts what the differences would take in FP64); the same with every further first
+// difference, of the state and of the stored differences, taken beforehand on the integer pipe and read from a table (2,
+// 3: the right-hand-side kernels).  The second
 // differences stay in FP64: along the azimuth near the axis or a pole their rounding, at 2^-53 of f against
 // f'' dxx^2, is multiplied by 1/(dxx S)^2, so another rounding would show in the result.
 // The table lies in the thread's local memory (2) or in shared memory, [entry][lane] (3).  The constraints, which
@@ -1623,7 +1625,8 @@ struct FxD1 {
     }
 };
 
-// a - b, rounded as the FP64 subtraction rounds it
+// a - b, exact where the two lie within 9 binades and otherwise off by up to 2^-61 of the larger, then rounded to
+// nearest, ties away from zero (the FP64 subtraction rounds ties to even)
 __device__ __forceinline__ double fx_sub(double a, double b)
 {
     const fx_u64 ba = (fx_u64)__double_as_longlong(a), bb = (fx_u64)__double_as_longlong(b);
@@ -1754,7 +1757,8 @@ __device__ __forceinline__ void mom_table(const PointIn& P, double raw[DiagIx::N
     diag_table<ORD, h | a | 1u << G_CF | 1u << G_TRK>(P.y, P.T, P.st, false, raw);
 }
 
-// Adds the upwinded advection and the dissipation to the 24 right-hand sides of rhs_core.
+// Adds the upwinded advection and the dissipation to the 24 right-hand sides of rhs_core (host checks; the kernels take
+// the sums ahead of rhs_core).
 template <int AX, int ORD>
 __device__ __forceinline__ void add_adv_ko(const double* y, long T, const long st[3], long ox, const double D[3],
                                            double sigma_metric, double sigma_gauge, double k[NGF])

@@ -8,9 +8,10 @@
 //
 // Values enter as m = mantissa * 2^SH >> (E - e): integers in units of 2^(E - 1075 - SH), where E is the
 // largest biased exponent of the sum's values and SH the guard bits below the mantissa.  Values within
-// SH binades of the largest enter exactly; the rest are off by less than one unit, 2^-(53 + SH)
+// SH binades of the largest enter exactly; the rest are off by less than one unit, at most 2^-(52 + SH)
 // of the largest (an FP64 sum rounds at 2^-53 of each partial sum).  Zeros and values more than
-// 64 binades down enter as 0.  The callers keep E away from both ends of the exponent range and
+// 64 binades down enter as 0.  Results are rounded to nearest, ties away from zero, the same for either sign.  The
+// callers keep E away from both ends of the exponent range and
 // leave sums outside to FP64 arithmetic, which also handles infinities and NaNs.
 #pragma once
 

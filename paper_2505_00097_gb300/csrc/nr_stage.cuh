@@ -267,7 +267,8 @@ __host__ __device__ inline long d1_points(const GridK& G)
 // The first differences alone would keep the FP64 pipe busy and the integer pipe idle: five of the eleven
 // gridfunctions are differenced in FP64, six on the integer pipe (two and three of each five).  k_d1 of
 // 256x2x512: 22.0 -> 15.5 us (all on the integer pipe: 19.6), 8th order 50.0 -> 30.2 (31.1), 192x96x192 8th order, two
-// axes, 1.30 -> 0.67 ms (0.91).
+// axes, 1.30 -> 0.67 ms (0.91).  On the smallest grids the integer sums' latency costs up to 1 % of a step (four steps of
+// 64x16x2: 1093 -> 1104 us); no rule on sizes is possible, since a partition must store the whole grid's bits.
 __host__ __device__ constexpr bool d1_integer(int q) { return q % 5 >= 2; }
 
 // point t of that region: raw first differences along axis 0 (and 1) of the N_D1
