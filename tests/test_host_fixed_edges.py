@@ -155,3 +155,17 @@ def test_negated_values_give_the_negated_sum(lib, order, ax):
         for o, s in zip(out, (1.0, -1.0)):
             lib.fixed_advko(ax, order, _p(np.ascontiguousarray(s * f)), _p(vet), _p(D), ctypes.c_double(0.3), _p(o), _p(np.empty(1)))
         assert out[0][0] == -out[1][0]
+
+
+def test_subtraction_bound_and_ties(lib):
+    """One rounding to nearest plus what the alignment cuts beyond 9 binades; ties away from zero, for either sign."""
+    rng = np.random.default_rng(23)
+    a = rng.uniform(0.5, 1, 4000) * rng.choice([-1.0, 1.0], 4000)
+    b = rng.uniform(0.5, 1, 4000) * rng.choice([-1.0, 1.0], 4000) * 2.0 ** rng.integers(-70, 1, 4000)
+    a[:4], b[:4] = (1.0, -1.0, 1.0, -1.0), (-2.0 ** -53, 2.0 ** -53, 2.0 ** -54, -2.0 ** -54)
+    out = np.empty(4000)
+    lib.fixed_sub(_p(a), _p(b), ctypes.c_long(4000), _p(out))
+    for x, y, o in zip(a, b, out):
+        exact, big = Fr(float(x)) - Fr(float(y)), max(abs(Fr(float(x))), abs(Fr(float(y))))
+        assert abs(Fr(float(o)) - exact) <= abs(exact) / 2 ** 53 + big / 2 ** 61
+    assert out[0] == 1.0 + 2.0 ** -52 and out[1] == -out[0] and out[2] == 1.0 and out[3] == -1.0
