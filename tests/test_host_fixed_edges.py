@@ -169,3 +169,32 @@ def test_subtraction_bound_and_ties(lib):
         exact, big = Fr(float(x)) - Fr(float(y)), max(abs(Fr(float(x))), abs(Fr(float(y))))
         assert abs(Fr(float(o)) - exact) <= abs(exact) / 2 ** 53 + big / 2 ** 61
     assert out[0] == 1.0 + 2.0 ** -52 and out[1] == -out[0] and out[2] == 1.0 and out[3] == -1.0
+
+
+@pytest.mark.parametrize("ax", [-1, 1, 2])
+@pytest.mark.parametrize("order", [4, 8])
+def test_the_fp64_sum_that_takes_values_outside_the_range(lib, order, ax):
+    """The merged FP64 stencil against rational arithmetic: at most 33 weights of up to four roundings each, summed in one
+    chain, so 40 roundings of the terms' magnitudes bound it."""
+    G = len(KO[order]) // 2
+    rng = np.random.default_rng(29 + order + ax)
+    for _ in range(60):
+        f = np.ascontiguousarray(rng.uniform(-1, 1, (11, 11, 11)))
+        vet, D, sigma = rng.uniform(-0.3, 0.3, 3), 10.0 ** rng.uniform(-1, 1, 3), 0.3
+        out, fp = np.empty(1), np.empty(1)
+        lib.fixed_advko(ax, order, _p(f), _p(vet), _p(D), ctypes.c_double(sigma), _p(out), _p(fp))
+        tot, mag = Fr(0), Fr(0)
+        for d in range(3):
+            at = lambda o: Fr(float(f[tuple(5 + (o if 2 - i == d else 0) for i in range(3))]))  # noqa: E731
+            u, k = Fr(float(abs(vet[d]) * D[d])), KC[order] * Fr(sigma) * Fr(float(D[d]))
+            if d == ax:
+                c = {4: 16, 8: 768}[order] * u + {4: 32, 8: 512}[order] * k
+                tot += c * (at(1) - at(0))
+                mag += c * (abs(at(1)) + abs(at(0)))
+                continue
+            s = 1 if vet[d] > 0 else -1
+            terms = [u * w * at(s * o) for o, w in UP[order].items()] + [k * w * at(o - G) for o, w in enumerate(KO[order])]
+            tot += sum(terms)
+            mag += sum(abs(t) for t in terms)
+        assert abs(Fr(float(fp[0])) - tot) <= 40 * mag / 2 ** 53
+        assert abs(Fr(float(out[0])) - tot) <= 40 * mag / 2 ** 53
