@@ -1,15 +1,18 @@
 """The launch shapes of the right-hand side (tiles spread over four warps, three or four blocks per SM; one point per
-thread, two or four blocks per SM) on sizes at the lines of the rule that chooses among them: one evaluation and
-two steps, bitwise against the same grid in a batch with a tile shape set, which always runs one point per thread.
+thread, two or four blocks per SM) on sizes at the lines of the rule that chooses among them: two steps, bitwise
+against the same grid in a batch with a tile shape set, which always runs one point per thread, and one evaluation of
+the right-hand side against the oracle.
 """
 import numpy as np
 import pytest
 
 torch = pytest.importorskip("torch")
 
+from oracle.oracle import Oracle  # noqa: E402
 from paper_2505_00097_gb300 import binding as B  # noqa: E402
 from paper_2505_00097_gb300 import build as BUILD  # noqa: E402
 from paper_2505_00097_gb300 import workloads as W  # noqa: E402
+from tests._common import assert_close  # noqa: E402
 
 pytestmark = pytest.mark.gpu
 
@@ -94,3 +97,23 @@ def test_a_batch_of_any_shape_computes_the_bits_of_its_grids(order, kind, per_sm
             g.close()
     for a, c in zip(out[:3], out[3:]):
         assert np.all(np.isfinite(a)) and np.array_equal(a, c)
+
+
+@pytest.mark.parametrize("per_sm", [2.8, 3.1, 4.3, 8.3, 13.0])
+@pytest.mark.parametrize("kind", sorted(KINDS))
+@pytest.mark.parametrize("order", [4, 8])
+def test_one_evaluation_of_every_shape_matches_the_oracle(order, kind, per_sm):
+    """1e-12 of the largest component of each tensor, as every right-hand-side parity test."""
+    sm = torch.cuda.get_device_properties(0).multi_processor_count
+    spec = KINDS[kind](int(32 * per_sm * sm))
+    if order == 8:
+        spec = dict(spec, NG=5, ko_sigma=KO8)
+    o = Oracle(spec)
+    y = W.random_state(o.n, seed=31, smooth=True)
+    o.inner_bc(y)
+    g = B.Grid(spec)
+    out = torch.zeros(y.size, dtype=torch.float64, device="cuda")
+    g.rhs(torch.from_numpy(y).cuda(), out)
+    torch.cuda.synchronize()
+    assert_close(out.cpu().numpy(), o.rhs(y), o.T, 1e-12, mask=o.interior_mask(), what=f"{kind} {order}")
+    g.close()
