@@ -317,7 +317,7 @@ int nr_dt_cfl(int coords, const int Nxx[3], const nr_params* params, double* dt_
  *     for batches of few points 32 consecutive points per item, whose difference
  *     sums four warps share).
  *   nr_batch_autotune: times one substage launch of each compiled tile shape
- *     and of the shared 32 points on the batch (it writes only the RK work
+ *     and, on batches of few points, of the shared 32 points (it writes only the RK work
  *     buffers, not the states), keeps the fastest and returns it, the latter as
  *     32x1 (synchronises).
  *   nr_batch_rk4_step, nr_batch_ssprk3_step: dts[ngrids] per-grid step sizes

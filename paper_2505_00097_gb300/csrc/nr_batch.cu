@@ -44,6 +44,7 @@ struct nr_batch {
                               // autotuner picks on the workloads
     bool few = false;         // at most two blocks of 128 points per SM (build_table)
     int n_sm = 0;
+    long items = 0;           // tiles of 32 points and outer blocks of all grids (RhsLoad)
     int total = 0;
     int total_d1 = 0;          // items of the first-difference pass
     BGrid* d_grids = nullptr;
@@ -257,6 +258,7 @@ static int nr_batch_create_body(nr_grid* const* grids, int ngrids, nr_batch** ou
         RhsLoad load;
         load.n_sm = b->n_sm = grids[0]->load.n_sm;
         for (int q = 0; q < ngrids; q++) load.add(grids[q]->K, grids[q]->n_outer);
+        b->items = load.tiles + load.outer;
         const RhsShape shape = rhs_shape(b->fam, b->ord, b->two_point, load);
         if (shape == RHS_SPREAD3) b->tile = kNumTiles;
         if (shape == RHS_SPREAD4) b->tile = kNumTiles + 1;
@@ -320,6 +322,8 @@ static int nr_batch_autotune_body(nr_batch* b, const double* dts, int* tile_x, i
     float best_t = 1e30f;
     int rc = NR_OK;
     for (int t = 0; t < kNumShapes && rc == NR_OK; t++) {
+        // beyond two rounds of four blocks per SM the spread shapes never won, and timing them takes the longest
+        if (kTiles[t].spread && b->items > 8L * b->n_sm) continue;
         b->tile = t;
         if ((rc = build_table(b, dts, b->table_ssp))) break;
         // stage 1 writes only the stage buffer and the accumulator: the state is untouched

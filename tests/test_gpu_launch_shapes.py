@@ -20,7 +20,7 @@ KO8 = [0.3] * 17 + [0.99] * 7
 KINDS = {
     "cyl_two_point": lambda n: W.sinh_cylindrical((33, 2, max(12, n // 66)), rho_max=30.0, z_max=30.0),
     "sph_two_point": lambda n: W.sinh_spherical((33, max(10, n // 66), 2)),
-    "sph_general": lambda n: W.sinh_spherical((33, 9, 2 * max(3, n // 594))),
+    "sph_general": lambda n: W.sinh_spherical((33, max(6, n // 792), 24)),
     "cyl_general": lambda n: W.sinh_cylindrical((33, 6, max(12, n // 198)), rho_max=30.0, z_max=30.0),
 }
 
