@@ -223,13 +223,15 @@ __host__ __device__ constexpr int d1gf(int q) { return q < 6 ? q : q == 6 ? G_CF
 // differences stay in FP64: along the azimuth near the axis or a pole their rounding, at 2^-53 of f against
 // f'' dxx^2, is multiplied by 1/(dxx S)^2, so another rounding would show in the result.
 // The table lies in the thread's local memory (2) or in shared memory, [entry][lane] (3).  The constraints, which
-// have no stored differences, keep every first and mixed difference that they use in a table of their own (4,
-// DiagIx).
-enum : int { SRC_INLINE = 0, SRC_STORED = 1, SRC_TABLE = 2, SRC_SHARED = 3, SRC_DIAG = 4 };
+// have no stored differences, keep every first and mixed difference that they use in a table of their own (DiagIx) in local
+// (4) or shared memory (5).
+enum : int { SRC_INLINE = 0, SRC_STORED = 1, SRC_TABLE = 2, SRC_SHARED = 3, SRC_DIAG = 4, SRC_DIAG_SHARED = 5 };
 template <int S>
 __host__ __device__ constexpr bool src_table() { return S == SRC_TABLE || S == SRC_SHARED; }
 template <int S>
-__host__ __device__ constexpr int src_stride() { return S == SRC_SHARED ? 32 : 1; }
+__host__ __device__ constexpr bool src_diag() { return S == SRC_DIAG || S == SRC_DIAG_SHARED; }
+template <int S>
+__host__ __device__ constexpr int src_stride() { return S == SRC_SHARED || S == SRC_DIAG_SHARED ? 32 : 1; }
 // Table index of each raw sum.  Per gridfunction with second derivatives (d1slot q): the first difference along the
 // last axis (AX < 0: axis 2; else the axis beside 0 and the two-point one), the mixed differences, and f_other -
 // f along a two-point axis; per gridfunction with first derivatives only (lambda 0..2, K: r = 0..3) the
@@ -281,7 +283,7 @@ __device__ __forceinline__ double hess(const double* f, const double* fx, const 
         constexpr int k = spi(KL), l = spj(KL);
         double m;
         if constexpr (src_table<S>()) m = rw[R::mix(q, KL) * src_stride<S>()];
-        else if constexpr (S == SRC_DIAG) m = rw[DiagIx::mix(q, KL)];
+        else if constexpr (src_diag<S>()) m = rw[DiagIx::mix(q, KL) * src_stride<S>()];
         else if constexpr (S == SRC_STORED && k == 0) m = d1r<ORD>(fx, st[l]);
         else if constexpr (S == SRC_STORED && AX < 0) m = d1r<ORD>(fy, st[l]);
         else m = mixr<ORD>(f, st[k], st[l]);
@@ -412,7 +414,7 @@ __device__ __forceinline__ double der1(const PointIn& P, int gf, int k)
 {
     if (k == AX) return 0.0;
     const int q = d1slot(gf);
-    if constexpr (S == SRC_DIAG) return P.g.D[k] * P.raw[DiagIx::d1(gf, k)];
+    if constexpr (src_diag<S>()) return P.g.D[k] * P.raw[DiagIx::d1(gf, k) * src_stride<S>()];
     if (S && q >= 0 && k == 0) return P.g.D[0] * ld(P.dx + (long)q * P.T);
     if (S && AX < 0 && q >= 0 && k == 1) return P.g.D[1] * ld(P.dy + (long)q * P.T);
     if (src_table<S>())
@@ -1722,39 +1724,43 @@ __device__ __forceinline__ double fx_mix(const double* f, long sa, long sb)
 }
 
 // the constraints' table of one point (DiagIx): first differences of the gridfunctions with their bit set in GFS and,
-// mixed, the mixed differences
+// mixed, the mixed differences; entries first, first + step, ... (mixed ones, then first differences), entry j into
+// raw[j * stride]
 template <int ORD, unsigned GFS>
-__device__ __forceinline__ void diag_table(const double* y, long T, const long st[3], bool mixed, double* raw)
+__device__ __forceinline__ void diag_table(const double* y, long T, const long st[3], bool mixed, double* raw, int stride,
+                                           int first, int step)
 {
+    if (mixed)
+#ifdef __CUDACC__
+#pragma unroll 1
+#endif
+        for (int j = first; j < 21; j += step) {
+            const int m = j % 3;   // (0,1), (0,2), (1,2)
+            raw[(51 + j) * stride] = fx_mix<ORD>(y + (long)d1gf(j / 3) * T, m == 2 ? st[1] : st[0], m == 0 ? st[1] : st[2]);
+        }
+    int e = mixed ? 21 : 0;
 #ifdef __CUDACC__
 #pragma unroll 1
 #endif
     for (int j = 0; j < 3 * G_VET; j++) {
         const int gf = j / 3, k = j % 3;
         if (!(GFS >> gf & 1)) continue;
-        raw[j] = fx_d1<ORD>(y + (long)gf * T, k == 0 ? st[0] : k == 1 ? st[1] : st[2]);
+        if (e++ % step != first) continue;
+        raw[j * stride] = fx_d1<ORD>(y + (long)gf * T, k == 0 ? st[0] : k == 1 ? st[1] : st[2]);
     }
-    if (mixed)
-#ifdef __CUDACC__
-#pragma unroll 1
-#endif
-        for (int j = 0; j < 21; j++) {
-            const int m = j % 3;   // (0,1), (0,2), (1,2)
-            raw[51 + j] = fx_mix<ORD>(y + (long)d1gf(j / 3) * T, m == 2 ? st[1] : st[0], m == 0 ? st[1] : st[2]);
-        }
 }
 // the tables that the Hamiltonian (h, W, lambda; K has no derivative in it) and the momentum constraint (h, a, W, K) read
 template <int ORD>
-__device__ __forceinline__ void ham_table(const PointIn& P, double raw[DiagIx::N])
+__device__ __forceinline__ void ham_table(const PointIn& P, double* raw, int stride = 1, int first = 0, int step = 1)
 {
     constexpr unsigned h = 0x3Fu << G_HDD, lam = 7u << G_LAM;
-    diag_table<ORD, h | 1u << G_CF | lam>(P.y, P.T, P.st, true, raw);
+    diag_table<ORD, h | 1u << G_CF | lam>(P.y, P.T, P.st, true, raw, stride, first, step);
 }
 template <int ORD>
-__device__ __forceinline__ void mom_table(const PointIn& P, double raw[DiagIx::N])
+__device__ __forceinline__ void mom_table(const PointIn& P, double* raw, int stride = 1, int first = 0, int step = 1)
 {
     constexpr unsigned h = 0x3Fu << G_HDD, a = 0x3Fu << G_ADD;
-    diag_table<ORD, h | a | 1u << G_CF | 1u << G_TRK>(P.y, P.T, P.st, false, raw);
+    diag_table<ORD, h | a | 1u << G_CF | 1u << G_TRK>(P.y, P.T, P.st, false, raw, stride, first, step);
 }
 
 // Adds the upwinded advection and the dissipation to the 24 right-hand sides of rhs_core (host checks; the kernels take

@@ -644,7 +644,13 @@ int nrk::grid_from_setup(HostSetup& H, const nr_params& P, nr_grid** out)
         std::vector<double> finf(P.f_inf, P.f_inf + NR_NGF), ws(P.wavespeed, P.wavespeed + NR_NGF);
         GridK& K = g->K;
         K = H.K;
-        g->nparts = ham_partials_needed(K);
+        cudaError_t e = cudaDeviceGetAttribute(&g->load.n_sm, cudaDevAttrMultiProcessorCount, g->device);
+        if (e != cudaSuccess) {
+            free_grid(g);
+            return fail(NR_ECUDA, "device attribute: %s", cudaGetErrorString(e));
+        }
+        g->load.add(K, g->n_outer);
+        g->nparts = ham_partials_needed(K, g->load.n_sm);
         if ((rc = dmalloc(g, &g->y, set)) || (rc = dmalloc(g, &g->ya, set)) || (rc = dmalloc(g, &g->yb, set)) ||
             (rc = dmalloc(g, &g->acc, set)) || (rc = dmalloc(g, &g->d1x, (size_t)N_D1 * G.T)) ||
             (rc = dmalloc(g, &g->d1y, K.ax < 0 ? (size_t)N_D1 * G.T : 1)) || (rc = dmalloc(g, &g->ax0, a0.size())) ||
@@ -660,7 +666,6 @@ int nrk::grid_from_setup(HostSetup& H, const nr_params& P, nr_grid** out)
         K.rfm.ax0 = g->ax0;
         K.rfm.ax1 = g->ax1;
         K.rfm.ax2 = g->ax2;
-        cudaError_t e = cudaSuccess;
         auto up = [&](void* d, const void* h, size_t b) {
             if (e == cudaSuccess && b) e = cudaMemcpy(d, h, b, cudaMemcpyHostToDevice);
         };
@@ -676,8 +681,6 @@ int nrk::grid_from_setup(HostSetup& H, const nr_params& P, nr_grid** out)
         if (e == cudaSuccess) e = cudaMemset(g->y, 0, sizeof(double) * set);
         if (e == cudaSuccess) e = cudaMemset(g->acc, 0, sizeof(double) * set);
         if (e == cudaSuccess) e = cudaStreamCreateWithFlags(&g->cap, cudaStreamNonBlocking);
-        if (e == cudaSuccess) e = cudaDeviceGetAttribute(&g->load.n_sm, cudaDevAttrMultiProcessorCount, g->device);
-        g->load.add(K, g->n_outer);
         if (e != cudaSuccess) {
             free_grid(g);
             return fail(NR_ECUDA, "grid upload: %s", cudaGetErrorString(e));
@@ -847,7 +850,7 @@ int nr_hamiltonian(nr_grid* g, const double* y_dev, double* H_dev, double* l2_ou
     if (!y_dev) CUDA_OR_FAIL(refresh_ghosts(g));
     const double* y = y_dev ? y_dev : g->y;
     if (H_dev) CUDA_OR_FAIL(cudaMemsetAsync(H_dev, 0, sizeof(double) * g->geo.T, g->stream));
-    CUDA_OR_FAIL(launch_ham(g->K, y, H_dev, g->P.h_rmin, g->P.h_rmax, g->partials, g->nparts, g->hres, g->stream));
+    CUDA_OR_FAIL(launch_ham(g->K, y, H_dev, g->P.h_rmin, g->P.h_rmax, g->partials, g->hres, g->load.n_sm, g->stream));
     if (l2_out || linf_out) {
         double r[3];
         CUDA_OR_FAIL(cudaMemcpyAsync(r, g->hres, sizeof r, cudaMemcpyDeviceToHost, g->stream));
@@ -865,7 +868,7 @@ int nr_momentum(nr_grid* g, const double* y_dev, double* M_dev, double* l2_out, 
     if (!y_dev) CUDA_OR_FAIL(refresh_ghosts(g));
     const double* y = y_dev ? y_dev : g->y;
     if (M_dev) CUDA_OR_FAIL(cudaMemsetAsync(M_dev, 0, sizeof(double) * 3 * g->geo.T, g->stream));
-    CUDA_OR_FAIL(launch_mom(g->K, y, M_dev, g->P.h_rmin, g->P.h_rmax, g->partials, g->nparts, g->hres, g->stream));
+    CUDA_OR_FAIL(launch_mom(g->K, y, M_dev, g->P.h_rmin, g->P.h_rmax, g->partials, g->hres, g->load.n_sm, g->stream));
     if (l2_out || linf_out) {
         double r[3];
         CUDA_OR_FAIL(cudaMemcpyAsync(r, g->hres, sizeof r, cudaMemcpyDeviceToHost, g->stream));

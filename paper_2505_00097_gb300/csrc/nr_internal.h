@@ -141,11 +141,12 @@ cudaError_t launch_compact(const GridK& G, const int* canon, long nc, const doub
 // ctr: perturbation counter per canonical point (NULL: its flat index in G)
 cudaError_t launch_bl(const GridK& G, const int* canon_idx, long ncanon, int np, const double* mxyz, double amp,
                       uint64_t seed, double* y, cudaStream_t s, const int* ctr = nullptr);
+// the constraints on a device of n_sm SMs; partials: ham_partials_needed(G, n_sm) blocks' norms
 cudaError_t launch_ham(const GridK& G, const double* y, double* H, double rmin, double rmax, double* partials,
-                       int nparts, double* result, cudaStream_t s);
+                       double* result, int n_sm, cudaStream_t s);
 cudaError_t launch_mom(const GridK& G, const double* y, double* M, double rmin, double rmax, double* partials,
-                       int nparts, double* result, cudaStream_t s);
-int ham_partials_needed(const GridK& G);
+                       double* result, int n_sm, cudaStream_t s);
+int ham_partials_needed(const GridK& G, int n_sm);
 cudaError_t launch_finite(const GridK& G, const double* y, int* flag, cudaStream_t s);
 // 64-bit digest of the 24 gridfunctions of y at the canonical points canon[0..nc) into *out; ctr: the
 // key of each point (NULL: its flat index in G)

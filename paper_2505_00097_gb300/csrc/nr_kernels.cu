@@ -97,10 +97,11 @@ __global__ void k_bl(GridK G, const int* __restrict__ canon, const int* __restri
 }
 
 // The constraints, one point per thread: the first and mixed differences on the integer pipe into a table in local
-// memory, then the FP64 part, which bounds them (as in k_rhs).  Six blocks per SM (80 registers): both constraints
-// with their norms on 256x2x512 in 751 us, against 792 / 876 / 1063 us with four, three, two, and 904 us with the
-// differences in FP64 (no limit on the registers).
-constexpr int HAM_THREADS = 128, HAM_BLOCKS = 6;
+// memory, then the FP64 part, which bounds them (as in k_rhs).  BPS blocks per SM: with six (80 registers) both
+// constraints with their norms take 751 us on 256x2x512, against 792 / 876 / 1063 us with four, three, two, and 904 us
+// with the differences in FP64 (no limit on the registers).  The Hamiltonian constraint takes three (168 registers, no
+// spills to speak of) where one round holds them (ham_shape).
+constexpr int HAM_THREADS = 128;
 
 // per-block partial norms (sum of squares, max, count) of a constraint, in a fixed order
 __device__ __forceinline__ void block_partials(double s2, double mx, double cnt, double* partials)
@@ -125,85 +126,98 @@ __device__ __forceinline__ void block_partials(double s2, double mx, double cnt,
     }
 }
 
-template <int FAM, int ORD>
-__global__ void __launch_bounds__(HAM_THREADS, HAM_BLOCKS) k_ham(GridK G, const double* __restrict__ y, double* H, double rmin,
-                                                      double rmax, double* partials)
+// interior point t (i0 fastest) of a constraint: padded indices, and the inputs but geometry and differences
+__device__ __forceinline__ PointIn constraint_point(const GridK& G, const double* __restrict__ y, long t, int p[3])
+{
+    const int i = (int)(t % G.N0), j = (int)(t / G.N0);
+    p[0] = i + G.NG;
+    p[1] = j % G.N1 + G.NG;
+    p[2] = j / G.N1 + G.NG;
+    return point_in<-1>(G, y, nullptr, nullptr, p[0], p[1], p[2]);
+}
+
+// the FP64 part of a constraint (MOM: momentum, Eq. Mconstraint, rescaled M^i; else Hamiltonian, Eq. Hconstraint) at one
+// point from the table P.raw, into out (1 or 3 gridfunctions, or NULL), and its share of the norms (of |M|)
+template <int FAM, int ORD, bool MOM, int S>
+__device__ __forceinline__ void constraint_value(const GridK& G, PointIn& P, const double* y, const int p[3], double* out,
+                                                 double rmin, double rmax, double& s2, double& mx, double& cnt)
+{
+    const long idx = P.y - y;
+    P.g = make_geo<FAM>(G, p[0], p[1], p[2]);
+    double v;
+    if constexpr (MOM) {
+        double Mv[3];
+        v = mom_core<FAM, ORD, S>(P, Mv);
+        if (out) {
+            out[idx] = Mv[0];
+            out[G.T + idx] = Mv[1];
+            out[2 * G.T + idx] = Mv[2];
+        }
+    } else {
+        v = ham_core<FAM, ORD, S>(P);
+        if (out) out[idx] = v;
+    }
+    double x[3];
+    cart_of(G, p[0], p[1], p[2], x);
+    const double r = sqrt(x[0] * x[0] + x[1] * x[1] + x[2] * x[2]);
+    if (r >= rmin && r <= rmax) {
+        s2 = v * v;
+        mx = fabs(v);
+        cnt = 1.0;
+    }
+}
+
+template <int FAM, int ORD, bool MOM>
+__device__ __forceinline__ void constraint_points(const GridK& G, const double* __restrict__ y, double* out, double rmin,
+                                                  double rmax, double* partials)
 {
     const long t = (long)blockIdx.x * HAM_THREADS + threadIdx.x;
-    const long nint = (long)G.N0 * G.N1 * G.N2;
     double s2 = 0.0, mx = 0.0, cnt = 0.0;
-    if (t < nint) {
-        const int i = (int)(t % G.N0), j = (int)(t / G.N0);
-        const int p0 = i + G.NG, p1 = j % G.N1 + G.NG, p2 = j / G.N1 + G.NG;
-        const long idx = p0 + (long)G.n0 * (p1 + (long)G.n1 * p2);
-        PointIn P;
-        P.y = y + idx;
-        P.T = G.T;
-        P.st[0] = 1;
-        P.st[1] = G.n0;
-        P.st[2] = (long)G.n0 * G.n1;
-        P.ox = 0;
-        P.dx = nullptr;
-        P.dy = nullptr;
+    if (t < (long)G.N0 * G.N1 * G.N2) {
+        int p[3];
+        PointIn P = constraint_point(G, y, t, p);
         double raw[DiagIx::N];
-        ham_table<ORD>(P, raw);
+        if constexpr (MOM) mom_table<ORD>(P, raw);
+        else ham_table<ORD>(P, raw);
         P.raw = raw;
-        P.g = make_geo<FAM>(G, p0, p1, p2);
-        const double h = ham_core<FAM, ORD, SRC_DIAG>(P);
-        if (H) H[idx] = h;
-        double x[3];
-        cart_of(G, p0, p1, p2, x);
-        const double r = sqrt(x[0] * x[0] + x[1] * x[1] + x[2] * x[2]);
-        if (r >= rmin && r <= rmax) {
-            s2 = h * h;
-            mx = fabs(h);
-            cnt = 1.0;
-        }
+        constraint_value<FAM, ORD, MOM, SRC_DIAG>(G, P, y, p, out, rmin, rmax, s2, mx, cnt);
     }
     block_partials(s2, mx, cnt, partials);
 }
-
-// momentum constraint (Eq. Mconstraint): rescaled M^i at interior points (M: 3 gridfunctions, or
-// NULL) and per-block partial norms of |M|
-template <int FAM, int ORD>
-__global__ void __launch_bounds__(HAM_THREADS, HAM_BLOCKS) k_mom(GridK G, const double* __restrict__ y, double* Mout, double rmin,
-                                                      double rmax, double* partials)
+template <int FAM, int ORD, int BPS>
+__global__ void __launch_bounds__(HAM_THREADS, BPS) k_ham(GridK G, const double* __restrict__ y, double* H, double rmin,
+                                                                 double rmax, double* partials)
 {
-    const long t = (long)blockIdx.x * HAM_THREADS + threadIdx.x;
-    const long nint = (long)G.N0 * G.N1 * G.N2;
+    constraint_points<FAM, ORD, false>(G, y, H, rmin, rmax, partials);
+}
+template <int FAM, int ORD>
+__global__ void __launch_bounds__(HAM_THREADS, 6) k_mom(GridK G, const double* __restrict__ y, double* M, double rmin,
+                                                                 double rmax, double* partials)
+{
+    constraint_points<FAM, ORD, true>(G, y, M, rmin, rmax, partials);
+}
+
+// The same on grids of few points, whose time is one warp's way through its tile: 32 consecutive points per block, the
+// differences divided among its warps, as in k_rhs_spread, and the same arithmetic per point.  BPS blocks per SM (168,
+// 128 or 80 registers).
+template <int FAM, int ORD, bool MOM, int BPS>
+__global__ void __launch_bounds__(32 * SPREAD_WARPS, BPS)
+    k_constraint_spread(GridK G, const double* __restrict__ y, double* out, double rmin, double rmax, double* partials)
+{
+    static_assert(HAM_THREADS == 32 * SPREAD_WARPS, "block_partials");
+    __shared__ double tab[DiagIx::N][32];
+    __shared__ int slot;
+    const int lane = threadIdx.x & 31, warp = threadIdx.x / 32;
+    const long n = (long)G.N0 * G.N1 * G.N2, t = (long)blockIdx.x * 32 + lane;
+    int p[3];
+    PointIn P = constraint_point(G, y, t < n ? t : n - 1, p);
+    if constexpr (MOM) mom_table<ORD>(P, &tab[0][lane], 32, warp, SPREAD_WARPS);
+    else ham_table<ORD>(P, &tab[0][lane], 32, warp, SPREAD_WARPS);
+    spread_slot(&slot);
     double s2 = 0.0, mx = 0.0, cnt = 0.0;
-    if (t < nint) {
-        const int i = (int)(t % G.N0), j = (int)(t / G.N0);
-        const int p0 = i + G.NG, p1 = j % G.N1 + G.NG, p2 = j / G.N1 + G.NG;
-        const long idx = p0 + (long)G.n0 * (p1 + (long)G.n1 * p2);
-        PointIn P;
-        P.y = y + idx;
-        P.T = G.T;
-        P.st[0] = 1;
-        P.st[1] = G.n0;
-        P.st[2] = (long)G.n0 * G.n1;
-        P.ox = 0;
-        P.dx = nullptr;
-        P.dy = nullptr;
-        double raw[DiagIx::N];
-        mom_table<ORD>(P, raw);
-        P.raw = raw;
-        P.g = make_geo<FAM>(G, p0, p1, p2);
-        double Mv[3];
-        const double m = mom_core<FAM, ORD, SRC_DIAG>(P, Mv);
-        if (Mout) {
-            Mout[idx] = Mv[0];
-            Mout[G.T + idx] = Mv[1];
-            Mout[2 * G.T + idx] = Mv[2];
-        }
-        double x[3];
-        cart_of(G, p0, p1, p2, x);
-        const double r = sqrt(x[0] * x[0] + x[1] * x[1] + x[2] * x[2]);
-        if (r >= rmin && r <= rmax) {
-            s2 = m * m;
-            mx = m;
-            cnt = 1.0;
-        }
+    if (warp == slot && t < n) {
+        P.raw = &tab[0][lane];
+        constraint_value<FAM, ORD, MOM, SRC_DIAG_SHARED>(G, P, y, p, out, rmin, rmax, s2, mx, cnt);
     }
     block_partials(s2, mx, cnt, partials);
 }
@@ -385,42 +399,84 @@ cudaError_t launch_bl(const GridK& G, const int* canon_idx, long ncanon, int np,
     return cudaGetLastError();
 }
 
-int ham_partials_needed(const GridK& G)
+// Launch shape of the constraints: spread tiles of 32 points while one round of three, four or six blocks per SM holds
+// them, else one point per thread.  us per call, spread with three / four / six, one point per thread with six, and with
+// all differences in FP64, 64x2xN cylindrical (the others alike); Hamiltonian constraint:
+//   256 tiles: 58 / 62 / 64, 88, 64;  8th order 80 / 82 / 88, 148, 117
+//   576: 103 / 68 / 72, 90, 64;  142 / 103 / 111, 148, 118
+//   896: 107 / 113 / 86, 119, 103;  164 / 157 / 137, 192, 211
+//   1216: 149 / 122 / 131, 123 (with three blocks per SM 115), 104;  220 / 181 / 184, 198 (185), 212
+//   1792: 198 / 173 / 154, 157 (146), 153;  305 / 257 / 240, 246 (228), 322
+// Momentum constraint, four / six: 256: 35 / 35, 43, 37; 896: 58 / 45, 58, 56; 1216: 62 / 68, 58, 56.
+enum HamShape { HAM_SPREAD3, HAM_SPREAD4, HAM_SPREAD6, HAM_POINTS3, HAM_POINTS6 };
+HamShape ham_shape(const GridK& G, int n_sm)
 {
-    const long nint = (long)G.N0 * G.N1 * G.N2;
-    return (int)((nint + HAM_THREADS - 1) / HAM_THREADS);
+    const long n = (long)G.N0 * G.N1 * G.N2, tiles = (n + 31) / 32, blocks = (n + HAM_THREADS - 1) / HAM_THREADS;
+    if (tiles <= 3L * n_sm) return HAM_SPREAD3;
+    if (tiles <= 4L * n_sm) return HAM_SPREAD4;
+    if (tiles <= 6L * n_sm) return HAM_SPREAD6;
+    return blocks <= 3L * n_sm ? HAM_POINTS3 : HAM_POINTS6;
+}
+
+int ham_partials_needed(const GridK& G, int n_sm)
+{
+    const long n = (long)G.N0 * G.N1 * G.N2, points = ham_shape(G, n_sm) <= HAM_SPREAD6 ? 32 : HAM_THREADS;
+    return (int)((n + points - 1) / points);
+}
+
+template <int FAM, int ORD>
+void launch_constraint(bool mom, const GridK& G, const double* y, double* out, double rmin, double rmax, double* partials,
+                       int nb, int n_sm, cudaStream_t s)
+{
+    switch (ham_shape(G, n_sm)) {
+    case HAM_SPREAD3:
+    case HAM_SPREAD4:
+        if (mom) k_constraint_spread<FAM, ORD, true, 4><<<nb, HAM_THREADS, 0, s>>>(G, y, out, rmin, rmax, partials);
+        else if (ham_shape(G, n_sm) == HAM_SPREAD3)
+            k_constraint_spread<FAM, ORD, false, 3><<<nb, HAM_THREADS, 0, s>>>(G, y, out, rmin, rmax, partials);
+        else k_constraint_spread<FAM, ORD, false, 4><<<nb, HAM_THREADS, 0, s>>>(G, y, out, rmin, rmax, partials);
+        break;
+    case HAM_SPREAD6:
+        if (mom) k_constraint_spread<FAM, ORD, true, 6><<<nb, HAM_THREADS, 0, s>>>(G, y, out, rmin, rmax, partials);
+        else k_constraint_spread<FAM, ORD, false, 6><<<nb, HAM_THREADS, 0, s>>>(G, y, out, rmin, rmax, partials);
+        break;
+    case HAM_POINTS3:
+        if (mom) k_mom<FAM, ORD><<<nb, HAM_THREADS, 0, s>>>(G, y, out, rmin, rmax, partials);
+        else k_ham<FAM, ORD, 3><<<nb, HAM_THREADS, 0, s>>>(G, y, out, rmin, rmax, partials);
+        break;
+    default:
+        if (mom) k_mom<FAM, ORD><<<nb, HAM_THREADS, 0, s>>>(G, y, out, rmin, rmax, partials);
+        else k_ham<FAM, ORD, 6><<<nb, HAM_THREADS, 0, s>>>(G, y, out, rmin, rmax, partials);
+    }
+}
+
+cudaError_t launch_constraints(bool mom, const GridK& G, const double* y, double* out, double rmin, double rmax,
+                               double* partials, double* result, int n_sm, cudaStream_t s)
+{
+    const int nparts = ham_partials_needed(G, n_sm);
+    if (G.fam == FAM_SPH) {
+        if (G.ord == 8) launch_constraint<FAM_SPH, 8>(mom, G, y, out, rmin, rmax, partials, nparts, n_sm, s);
+        else launch_constraint<FAM_SPH, 4>(mom, G, y, out, rmin, rmax, partials, nparts, n_sm, s);
+    } else {
+        if (G.ord == 8) launch_constraint<FAM_CYL, 8>(mom, G, y, out, rmin, rmax, partials, nparts, n_sm, s);
+        else launch_constraint<FAM_CYL, 4>(mom, G, y, out, rmin, rmax, partials, nparts, n_sm, s);
+    }
+    cudaError_t e = cudaGetLastError();
+    if (e != cudaSuccess) return e;
+    k_ham_reduce<<<1, 256, 0, s>>>(partials, nparts, result);
+    return cudaGetLastError();
 }
 
 cudaError_t launch_ham(const GridK& G, const double* y, double* H, double rmin, double rmax, double* partials,
-                       int nparts, double* result, cudaStream_t s)
+                       double* result, int n_sm, cudaStream_t s)
 {
-    if (G.fam == FAM_SPH) {
-        if (G.ord == 8) k_ham<FAM_SPH, 8><<<nparts, HAM_THREADS, 0, s>>>(G, y, H, rmin, rmax, partials);
-        else k_ham<FAM_SPH, 4><<<nparts, HAM_THREADS, 0, s>>>(G, y, H, rmin, rmax, partials);
-    } else {
-        if (G.ord == 8) k_ham<FAM_CYL, 8><<<nparts, HAM_THREADS, 0, s>>>(G, y, H, rmin, rmax, partials);
-        else k_ham<FAM_CYL, 4><<<nparts, HAM_THREADS, 0, s>>>(G, y, H, rmin, rmax, partials);
-    }
-    cudaError_t e = cudaGetLastError();
-    if (e != cudaSuccess) return e;
-    k_ham_reduce<<<1, 256, 0, s>>>(partials, nparts, result);
-    return cudaGetLastError();
+    return launch_constraints(false, G, y, H, rmin, rmax, partials, result, n_sm, s);
 }
 
 cudaError_t launch_mom(const GridK& G, const double* y, double* M, double rmin, double rmax, double* partials,
-                       int nparts, double* result, cudaStream_t s)
+                       double* result, int n_sm, cudaStream_t s)
 {
-    if (G.fam == FAM_SPH) {
-        if (G.ord == 8) k_mom<FAM_SPH, 8><<<nparts, HAM_THREADS, 0, s>>>(G, y, M, rmin, rmax, partials);
-        else k_mom<FAM_SPH, 4><<<nparts, HAM_THREADS, 0, s>>>(G, y, M, rmin, rmax, partials);
-    } else {
-        if (G.ord == 8) k_mom<FAM_CYL, 8><<<nparts, HAM_THREADS, 0, s>>>(G, y, M, rmin, rmax, partials);
-        else k_mom<FAM_CYL, 4><<<nparts, HAM_THREADS, 0, s>>>(G, y, M, rmin, rmax, partials);
-    }
-    cudaError_t e = cudaGetLastError();
-    if (e != cudaSuccess) return e;
-    k_ham_reduce<<<1, 256, 0, s>>>(partials, nparts, result);
-    return cudaGetLastError();
+    return launch_constraints(true, G, y, M, rmin, rmax, partials, result, n_sm, s);
 }
 
 cudaError_t launch_ham_reduce(const double* partials, int nparts, double* result, cudaStream_t s)

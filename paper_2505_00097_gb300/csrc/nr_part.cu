@@ -560,10 +560,16 @@ static int nr_part_create_body(int coords, const int Nxx[3], const nr_params* pa
                 return nrk_fail(NR_ECUDA, "partition set-up: %s", cudaGetErrorString(e));
             }
         }
+        // the partitions' kernels are parallel branches of the captured step
+        for (PartDev& d : s->p) s->load.add(d.K, d.n_outer);
+        if (cudaError_t e = cudaDeviceGetAttribute(&s->load.n_sm, cudaDevAttrMultiProcessorCount, s->device)) {
+            free_part(s);
+            return nrk_fail(NR_ECUDA, "device attribute: %s", cudaGetErrorString(e));
+        }
         s->part_off.assign(s->p.size(), 0);
         for (size_t q = 0; q < s->p.size(); q++) {
             s->part_off[q] = s->nparts_total;
-            s->nparts_total += ham_partials_needed(s->p[q].K);
+            s->nparts_total += ham_partials_needed(s->p[q].K, s->load.n_sm);
         }
         if ((rc = pmalloc(s, &s->partials, 3 * (size_t)s->nparts_total)) || (rc = pmalloc(s, &s->hres, 3))) {
             free_part(s);
@@ -584,10 +590,7 @@ static int nr_part_create_body(int coords, const int Nxx[3], const nr_params* pa
                     return rc;
                 }
             }
-        // the partitions' kernels are parallel branches of the captured step
-        for (PartDev& d : s->p) s->load.add(d.K, d.n_outer);
-        cudaError_t e = cudaDeviceGetAttribute(&s->load.n_sm, cudaDevAttrMultiProcessorCount, s->device);
-        if (e == cudaSuccess) e = cudaStreamCreateWithFlags(&s->cap, cudaStreamNonBlocking);
+        cudaError_t e = cudaStreamCreateWithFlags(&s->cap, cudaStreamNonBlocking);
         if (e == cudaSuccess) e = cudaEventCreateWithFlags(&s->fork, cudaEventDisableTiming);
         s->pstream.assign(s->p.size(), nullptr);
         s->pevent.assign(s->p.size(), nullptr);
@@ -739,8 +742,8 @@ static int nr_part_hamiltonian_body(nr_part* s, double* l2_out, double* linf_out
     // it also runs writes a scratch result nobody reads), then one reduction over all of them
     for (size_t q = 0; q < s->p.size(); q++) {
         PartDev& d = s->p[q];
-        PCUDA(launch_ham(d.K, d.y, nullptr, s->P.h_rmin, s->P.h_rmax, s->partials + 3 * (size_t)s->part_off[q],
-                         ham_partials_needed(d.K), s->hres, s->stream));
+        PCUDA(launch_ham(d.K, d.y, nullptr, s->P.h_rmin, s->P.h_rmax, s->partials + 3 * (size_t)s->part_off[q], s->hres,
+                         s->load.n_sm, s->stream));
     }
     PCUDA(launch_ham_reduce(s->partials, s->nparts_total, s->hres, s->stream));
     double r[3];

@@ -1,7 +1,7 @@
 // Test harness: the per-point bodies of the kernels (nr_stage.cuh), compiled for the host with g++ and run over a
 // small grid as the kernels run them: the stored first differences (d1_point), then rhs_point_stage per point
 // (k_rhs, k_batch_stage) or rhs_spread_stage per tile of 32 points by four emulated warps (k_rhs_spread); the
-// constraints from their tables as k_ham and k_mom fill them.
+// constraints from their tables as k_ham and k_mom, and k_constraint_spread's warps, fill them.
 #include <cmath>
 #include <cstring>
 #include <vector>
@@ -112,26 +112,37 @@ void rhs(const GridK& G, const double* y, double* out, bool spread)
     }
 }
 
+// at one point, from a table of stride 1 filled at once, or (spread) of stride 32 filled by four warps in turn
+template <int FAM, int ORD, int S>
+void constraint_at(const GridK& G, PointIn P, const double* y, double* out, int p0, int p1, int p2, bool momentum)
+{
+    constexpr int stride = src_stride<S>(), warps = S == SRC_DIAG_SHARED ? SPREAD_WARPS : 1;
+    const long idx = P.y - y;
+    std::vector<double> raw(DiagIx::N * stride, NAN);
+    for (int w = 0; w < warps; w++) {
+        if (momentum) mom_table<ORD>(P, raw.data() + stride - 1, stride, w, warps);
+        else ham_table<ORD>(P, raw.data() + stride - 1, stride, w, warps);
+    }
+    P.raw = raw.data() + stride - 1;
+    P.g = make_geo<FAM>(G, p0, p1, p2);
+    if (momentum) {
+        double M[3];
+        mom_core<FAM, ORD, S>(P, M);
+        for (int q = 0; q < 3; q++) out[q * G.T + idx] = M[q];
+    } else {
+        out[idx] = ham_core<FAM, ORD, S>(P);
+    }
+}
+
 template <int FAM, int ORD>
-void constraint(const GridK& G, const double* y, double* out, bool momentum)
+void constraint(const GridK& G, const double* y, double* out, bool momentum, bool spread)
 {
     for (int p2 = G.NG; p2 < G.NG + G.N2; p2++)
         for (int p1 = G.NG; p1 < G.NG + G.N1; p1++)
             for (int p0 = G.NG; p0 < G.NG + G.N0; p0++) {
-                PointIn P = point_in<-1>(G, y, nullptr, nullptr, p0, p1, p2);
-                const long idx = P.y - y;
-                std::vector<double> raw(DiagIx::N, NAN);
-                if (momentum) mom_table<ORD>(P, raw.data());
-                else ham_table<ORD>(P, raw.data());
-                P.raw = raw.data();
-                P.g = make_geo<FAM>(G, p0, p1, p2);
-                if (momentum) {
-                    double M[3];
-                    mom_core<FAM, ORD, SRC_DIAG>(P, M);
-                    for (int q = 0; q < 3; q++) out[q * G.T + idx] = M[q];
-                } else {
-                    out[idx] = ham_core<FAM, ORD, SRC_DIAG>(P);
-                }
+                const PointIn P = point_in<-1>(G, y, nullptr, nullptr, p0, p1, p2);
+                if (spread) constraint_at<FAM, ORD, SRC_DIAG_SHARED>(G, P, y, out, p0, p1, p2, momentum);
+                else constraint_at<FAM, ORD, SRC_DIAG>(G, P, y, out, p0, p1, p2, momentum);
             }
 }
 
@@ -143,8 +154,8 @@ void run(int coords, const int* N, const double* ampl, const double* sinhw, cons
     make_grid<ORD>(H, coords, N, ampl, sinhw, sigma, eta);
     const GridK& G = H.G;
     if (which >= 2) {
-        if (G.fam == FAM_CYL) constraint<FAM_CYL, ORD>(G, y, out, which == 3);
-        else constraint<FAM_SPH, ORD>(G, y, out, which == 3);
+        if (G.fam == FAM_CYL) constraint<FAM_CYL, ORD>(G, y, out, which % 2 == 1, which >= 4);
+        else constraint<FAM_SPH, ORD>(G, y, out, which % 2 == 1, which >= 4);
     } else if (G.fam == FAM_CYL) {
         if (G.ax == 1) rhs<FAM_CYL, 1, ORD>(G, y, out, which == 1);
         else rhs<FAM_CYL, -1, ORD>(G, y, out, which == 1);
@@ -157,7 +168,7 @@ void run(int coords, const int* N, const double* ampl, const double* sinhw, cons
 }  // namespace
 
 // which: 0 the right-hand side as k_rhs computes it, 1 as k_rhs_spread, 2 the Hamiltonian constraint, 3 the momentum
-// constraint.  sigma: the dissipation strength per gridfunction (metric at 0, gauge at G_VET).
+// constraint, 4 and 5 the same as k_constraint_spread.  sigma: the dissipation strength per gridfunction (metric at 0, gauge at G_VET).
 extern "C" void stage_point(int coords, const int* N, const double* ampl, const double* sinhw, const double* sigma, double eta,
                             const double* y, double* out, int which, int ng)
 {

@@ -117,3 +117,30 @@ def test_one_evaluation_of_every_shape_matches_the_oracle(order, kind, per_sm):
     torch.cuda.synchronize()
     assert_close(out.cpu().numpy(), o.rhs(y), o.T, 1e-12, mask=o.interior_mask(), what=f"{kind} {order}")
     g.close()
+
+
+# one round of three, four and six spread blocks per SM, one of three blocks of 128 points, and more
+@pytest.mark.parametrize("per_sm", [0.2, 2.9, 3.6, 5.5, 8.0, 13.0])
+@pytest.mark.parametrize("kind", ["cyl_two_point", "sph_general"])
+@pytest.mark.parametrize("order", [4, 8])
+def test_the_constraints_of_every_shape_match_the_oracle(order, kind, per_sm):
+    """Values to 1e-12 of the largest, norms to 1e-10, as every parity test of the constraints."""
+    sm = torch.cuda.get_device_properties(0).multi_processor_count
+    spec = KINDS[kind](int(32 * per_sm * sm))
+    if order == 8:
+        spec = dict(spec, NG=5, ko_sigma=KO8)
+    o = Oracle(spec)
+    y = W.random_state(o.n, seed=41, smooth=True)
+    o.inner_bc(y)
+    m = o.interior_mask()
+    g = B.Grid(spec)
+    yd = torch.from_numpy(y).cuda()
+    for comps, fn, ref in ((1, g.hamiltonian, o.hamiltonian(y)), (3, g.momentum, o.momentum(y))):
+        out = torch.zeros(comps * o.T, dtype=torch.float64, device="cuda")
+        norms = fn(yd, out)
+        torch.cuda.synchronize()
+        got, want = out.cpu().numpy().reshape(comps, o.T)[:, m], np.asarray(ref[0]).reshape(comps, o.T)[:, m]
+        assert np.abs(got - want).max() <= 1e-12 * np.abs(want).max()
+        for a, b in zip(norms, ref[-3:-1]):   # l2, linf
+            assert abs(a - b) <= 1e-10 * abs(b)
+    g.close()

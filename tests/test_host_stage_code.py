@@ -99,6 +99,9 @@ def test_constraint_bodies_match_the_oracle(lib, name, spec):
     ref = o.momentum(y)[0]
     got = _run(lib, spec, y, MOM, 3 * o.T).reshape(3, o.T)
     assert np.abs(got[:, m] - ref[:, m]).max() <= 1e-12 * np.abs(ref[:, m]).max()
+    # the table divided among four warps holds the same sums
+    assert np.array_equal(_run(lib, spec, y, HAM + 2, o.T), _run(lib, spec, y, HAM, o.T))
+    assert np.array_equal(_run(lib, spec, y, MOM + 2, 3 * o.T).reshape(3, o.T), got)
 
 
 SPH, CYL = 0, 1
