@@ -1738,14 +1738,17 @@ __device__ __forceinline__ void diag_table(const double* y, long T, const long s
             const int m = j % 3;   // (0,1), (0,2), (1,2)
             raw[(51 + j) * stride] = fx_mix<ORD>(y + (long)d1gf(j / 3) * T, m == 2 ? st[1] : st[0], m == 0 ? st[1] : st[2]);
         }
+    // gridfunctions 0 .. last - 1; without a gap among them and a division among warps the loop has nothing to test
+    constexpr int last = GFS >> G_LAM ? G_VET : G_LAM;
+    constexpr bool dense = GFS == (1u << last) - 1;
     int e = mixed ? 21 : 0;
 #ifdef __CUDACC__
 #pragma unroll 1
 #endif
-    for (int j = 0; j < 3 * G_VET; j++) {
+    for (int j = 0; j < 3 * last; j++) {
         const int gf = j / 3, k = j % 3;
-        if (!(GFS >> gf & 1)) continue;
-        if (e++ % step != first) continue;
+        if (!dense && !(GFS >> gf & 1)) continue;
+        if (step > 1 && e++ % step != first) continue;
         raw[j * stride] = fx_d1<ORD>(y + (long)gf * T, k == 0 ? st[0] : k == 1 ? st[1] : st[2]);
     }
 }
