@@ -14,13 +14,13 @@ namespace nrk {
 // ones with BPS = 4, the last ones with BPS = 2, whose tiles then fill whole SMs and leave the light outer blocks
 // beside them.
 //
-// Bound: the FP64 pipe (2 lanes a cycle per SM: 16 to 20 cycles per warp instruction), with the difference sums on the
-// integer pipe beside it (fixed_sum.cuh).  A warp does its integer passes first and its FP64 part after
-// them; four blocks per SM (128 registers, 3 to 5 KB of spills) keep one warp of each scheduler in its FP64 part nearly
-// always: 640 us per right-hand side on 256x2x512 when that was chosen, against 664 us with three (168 registers); two
-// (255 registers, no spills) were 10 % slower.  All in FP64 arithmetic, two per scheduler, 865 us, now 636; 8th order on
-// the same grid 1137 -> 744 us; 192x96x192 spherical 15.66 -> 10.47 ms (4th), 23.2 -> 12.9 ms (8th).  FP64 pipe 81 % active.  Where no scheduler gets more than two
-// warps, the 255 registers are the faster ones (rhs_shape).
+// Bound: the FP64 pipe (2 lanes a cycle per SM: 16 to 20 cycles per warp instruction), 81 % active on 256x2x512, with
+// the difference sums on the integer pipe beside it (fixed_sum.cuh).  A warp does its integer passes first and its
+// FP64 part after them; four blocks per SM (128 registers, 3 to 5 KB of spills) keep one warp of each scheduler in its
+// FP64 part nearly always: 640 us per right-hand side on 256x2x512 when that was chosen, against 664 us with three
+// (168 registers); two (255 registers, no spills) were 10 % slower.  All in FP64 arithmetic, two per scheduler, 865
+// us, now 636; 8th order on the same grid 1137 -> 744 us; 192x96x192 spherical 15.66 -> 10.47 ms (4th), 23.2 -> 12.9 ms
+// (8th).  Where no scheduler gets more than two warps, the 255 registers are the faster ones (rhs_shape).
 constexpr int RHS_WARPS = 4;
 template <int FAM, int AX, int ORD, int BPS>
 __global__ void __launch_bounds__(32 * RHS_WARPS, BPS)
